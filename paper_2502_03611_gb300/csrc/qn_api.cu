@@ -124,6 +124,7 @@ struct qn_ctx {
     int split_layout;     // 1: the last residual wrote its planes in split / folded order
     int last_split;       // 1: the last shifted inverse used the split products
     int f64_split;        // FP64 path: reflection-split FP64 products (FD Dirichlet / Neumann)
+    F64TcPlan *f64tc;     // FP64 path: the products on the tensor cores (nullptr: on the FP64 pipe)
     __nv_bfloat16 *bf_hi, *bf_lo, *bb_hi, *bb_lo;   // [P][P/2] forward / backward matrices
     // six-product backward level (QN_PREC_BF16X6): the third BF16 level of the two working
     // buffers and of the backward matrix; x6 = 1 while the solves use it
@@ -236,6 +237,28 @@ extern "C" int qn_version(void) { return 10400; }
 
 extern "C" const char *qn_last_error(void) { return g_err; }
 
+// sin(pi q / N) and cos(pi q / N) for integers 0 <= q < 2N, reduced on the integers to an
+// argument of at most pi/4: correct to about an ulp, and equal up to sign at mirrored
+// arguments, so that the eigenvector matrices have their reflection symmetry exactly.
+static double sin_ratio(long long q, long long N);
+
+static double cos_ratio(long long q, long long N) {
+    const double pi = 3.14159265358979323846;
+    if (q > N) q = 2 * N - q;                              // cos(2 pi - t) = cos t
+    if (2 * q > N) return -cos_ratio(N - q, N);            // cos(pi - t) = -cos t
+    if (2 * q == N) return 0.0;
+    if (4 * q > N) return sin(pi * (double)(N - 2 * q) / (double)(2 * N));   // sin(pi/2 - t)
+    return cos(pi * (double)q / (double)N);
+}
+
+static double sin_ratio(long long q, long long N) {
+    const double pi = 3.14159265358979323846;
+    if (q > N) return -sin_ratio(2 * N - q, N);            // sin(2 pi - t) = -sin t
+    if (2 * q > N) q = N - q;                              // sin(pi - t) = sin t
+    if (4 * q > N) return cos(pi * (double)(N - 2 * q) / (double)(2 * N));
+    return sin(pi * (double)q / (double)N);
+}
+
 extern "C" int qn_setup_1d_eig(int n, double h, int bc, double *S, double *S_inv, double *lam) {
     if (n < 1 || n > 65536 || (bc == QN_BC_NEUMANN && n < 2)) {
         set_error("qn_setup_1d_eig: n=%d out of range", n);
@@ -264,9 +287,7 @@ extern "C" int qn_setup_1d_eig(int n, double h, int bc, double *S, double *S_inv
             const double w = (j == 0 || j == n - 1) ? 0.5 : 1.0;
             for (int k = 0; k < n; ++k) {
                 const double ck = (k == 0 || k == n - 1) ? (double)(n - 1) : 0.5 * (n - 1);
-                // cos(j k pi t) with the product reduced mod 2(n-1)
-                const long long jk = ((long long)j * k) % (2LL * (n - 1));
-                const double v = cos(pi * (double)jk * t) / sqrt(ck);
+                const double v = cos_ratio(((long long)j * k) % (2LL * (n - 1)), n - 1) / sqrt(ck);
                 if (S) S[(size_t)j * n + k] = v;
                 if (S_inv) S_inv[(size_t)k * n + j] = w * v;
             }
@@ -281,9 +302,7 @@ extern "C" int qn_setup_1d_eig(int n, double h, int bc, double *S, double *S_inv
     }
     for (int j = 1; j <= n; ++j) {
         for (int k = 1; k <= n; ++k) {
-            // sin(j k pi h) with the product reduced mod 2(n+1) for accuracy
-            const long long jk = ((long long)j * k) % (2LL * (n + 1));
-            const double v = scale * sin(pi * (double)jk * hh);
+            const double v = scale * sin_ratio(((long long)j * k) % (2LL * (n + 1)), n + 1);
             if (S) S[(size_t)(j - 1) * n + (k - 1)] = v;
             if (S_inv) S_inv[(size_t)(j - 1) * n + (k - 1)] = v;   // symmetric orthogonal
         }
@@ -347,6 +366,7 @@ static void ctx_free(qn_ctx *c) {
     cudaFree(c->dU);
     cudaFree(c->df);
     if (c->plan) tc_plan_destroy(c->plan);
+    f64tc_destroy(c->f64tc);
     if (c->prof) {
         for (auto &r : *c->prof) {
             cudaEventDestroy(r.a);
@@ -585,6 +605,13 @@ extern "C" int qn_ctx_create(const qn_problem *p, qn_ctx **out) {
         // products use; the numerical (Robin, spectral-element) ones need not
         const char *es = getenv("QN_SPLIT");
         c->f64_split = (es ? (atoi(es) != 0) : true) && p->sem_k == 0 && p->bc != QN_BC_ROBIN;
+        if (f64tc_pays(n, c->dim)) {
+            rc = f64tc_create(&c->f64tc, n, c->dim, c->f64_split, c->S64, c->Si64, c->num_sms);
+            if (rc != QN_OK) {
+                ctx_free(c);
+                return rc;
+            }
+        }
     } else {
         if (!tc_supported(c->device)) {
             set_error("qn_ctx_create: QN_PREC_BF16X3 needs an sm_103 (tcgen05) device");
@@ -903,12 +930,17 @@ static int enqueue_inverse(qn_ctx *c, const double *r0, double *target, bool upd
             g.K = c->n;
             g.N = c->n;
             g.Mtot = (d == 3) ? c->n * c->n : c->n;
-            g.split = c->f64_split ? (forward ? 1 : 2) : 0;
             c->last_split = c->f64_split;
             const double *A = (i == 0 && r0 != nullptr) ? r0 : c->w64[cur];
             const double *B = forward ? c->Si64 : c->S64;
             double *o = last ? target : c->w64[next];
-            rc = launch_modeprod_f64(A, B, o, g, epi, e, s);
+            if (c->f64tc != nullptr) {
+                int nl = 1;
+                rc = launch_modeprod_f64tc(c->f64tc, forward, A, o, epi, e, s, &nl);
+                c->launches += nl - 1;
+            } else {
+                rc = launch_modeprod_f64(A, B, o, g, epi, e, s);
+            }
         } else {
             rc = launch_modeprod_tc(c->plan, cur, last ? -1 : next, forward, epi, e, s);
         }

@@ -116,7 +116,6 @@ struct GemmShape {
     int n;      // logical extent per axis
     int P;      // padded extent per axis (split path), = n for FP64
     int dim;
-    int split = 0;   // FP64 products: 0 dense, 1 forward / 2 backward reflection split
 };
 
 // ---- launchers (implemented in the .cu files) ---------------------------------
@@ -192,6 +191,16 @@ int launch_split_pad(const double *r, int n, int P, int dim, __nv_bfloat16 *hi, 
                      int grid, cudaStream_t s);
 int launch_modeprod_f64(const double *A, const double *B, double *out, const GemmShape &g,
                         Epi epi, const EpiArgs &e, cudaStream_t s);
+
+// FP64 products from integer digits on the tensor cores (qn_modeprod_f64tc.cu). split: the
+// reflection-split form (S, S^{-1} with the mirror symmetry); S, Si: device, n x n.
+struct F64TcPlan;
+bool f64tc_pays(int n, int dim);   // false: the FP64-pipe kernel is faster at this size
+int f64tc_create(F64TcPlan **out, int n, int dim, int split, const double *S, const double *Si, int num_sms);
+void f64tc_destroy(F64TcPlan *p);
+// As launch_modeprod_f64; forward selects S^{-1}. *launches: kernels launched.
+int launch_modeprod_f64tc(const F64TcPlan *p, bool forward, const double *A, double *out, Epi epi, const EpiArgs &e,
+                          cudaStream_t s, int *launches);
 
 // ---- tcgen05 split-precision mode products ------------------------------------------
 // One group = one GEMM out[k][m] = sum_j A[m][j] B[k][j] (one mode product of
@@ -272,6 +281,8 @@ int launch_modeprod_tc_grouped(const TcGroup *groups, const TcTile *tiles, int n
 // Encode a 2-D BF16 tensor map [outer][inner] with a (box_inner x box_outer) box.
 int tc_encode_2d(CUtensorMap *m, const void *ptr, uint64_t inner, uint64_t outer, uint32_t box_inner,
                  uint32_t box_outer, int BK);
+int tc_encode_tiled(CUtensorMap *m, CUtensorMapDataType type, int rank, const void *ptr, const cuuint64_t *dims,
+                    const cuuint64_t *strides, const cuuint32_t *box, CUtensorMapSwizzle swizzle);
 size_t tc_smem_bytes(int BK, int stages);
 int tc_set_attributes();
 int tc_stages(int BK);

@@ -80,7 +80,6 @@ constexpr int kEpiParts = kEpiWarps / 4;            // column ranges per quadran
 constexpr int kChunk = 16;                          // accumulator columns per TMEM load
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kMaxStages = 8;
-constexpr uint64_t kTimeoutNs = 2000000000ull;
 constexpr uint32_t kCtrlBytes = 512;
 constexpr uint32_t kTmemCols = 2 * BN_MAX;         // two accumulators of BN_MAX FP32 columns
 
@@ -95,29 +94,8 @@ __host__ __device__ constexpr int bn_slot(int mode) { return mode == 2 ? 128 : B
 // no MMA was issued and the other stages' loads are drained.
 __device__ int g_tc_withhold = 0;
 
-// Wait for `parity` on `bar`; false on timeout or when another role aborted.
-__device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile int *abort_flag,
-                                         int *err) {
-    if (ptx::mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = ptx::globaltimer();
-    while (true) {
-        if (ptx::mbar_try_wait(bar, parity)) return true;
-        if (*abort_flag) return false;
-        if (ptx::globaltimer() - t0 > kTimeoutNs) {
-            *abort_flag = 1;
-            atomicExch(err, QN_ETIMEOUT);
-            return false;
-        }
-    }
-}
-
-// Bounded wait that ignores the abort flag (used while draining after an abort).
-__device__ __forceinline__ void drain_bar(uint32_t bar, uint32_t parity) {
-    const uint64_t t0 = ptx::globaltimer();
-    while (!ptx::mbar_try_wait(bar, parity)) {
-        if (ptx::globaltimer() - t0 > kTimeoutNs) return;
-    }
-}
+using ptx::drain_bar;
+using ptx::wait_bar;
 
 __device__ __forceinline__ void split_store(float v, __nv_bfloat16 *hi, __nv_bfloat16 *lo, int o) {
     const __nv_bfloat16 h = __float2bfloat16_rn(v);
@@ -604,27 +582,32 @@ static PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
     return fn;
 }
 
-int tc_encode_2d(CUtensorMap *m, const void *ptr, uint64_t inner, uint64_t outer, uint32_t box_inner,
-                 uint32_t box_outer, int BK) {
+int tc_encode_tiled(CUtensorMap *m, CUtensorMapDataType type, int rank, const void *ptr, const cuuint64_t *dims,
+                    const cuuint64_t *strides, const cuuint32_t *box, CUtensorMapSwizzle swizzle) {
     PFN_cuTensorMapEncodeTiled_v12000 enc = get_encode();
     if (!enc) {
         set_error("cuTensorMapEncodeTiled unavailable from the driver");
         return QN_ECUDA;
     }
-    cuuint64_t dims[2] = {inner, outer};
-    cuuint64_t strides[1] = {inner * 2};
-    cuuint32_t box[2] = {box_inner, box_outer};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box,
-                     estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                     BK == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
-                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    const cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = enc(m, type, (cuuint32_t)rank, const_cast<void *>(ptr), dims, strides, box, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
-        set_error("cuTensorMapEncodeTiled failed (%d) for %llux%llu box %ux%u", (int)r,
-                  (unsigned long long)inner, (unsigned long long)outer, box_inner, box_outer);
+        set_error("cuTensorMapEncodeTiled failed (%d) for %llux%llu box %ux%u", (int)r, (unsigned long long)dims[0],
+                  (unsigned long long)dims[1], box[0], box[1]);
         return QN_ECUDA;
     }
     return QN_OK;
+}
+
+int tc_encode_2d(CUtensorMap *m, const void *ptr, uint64_t inner, uint64_t outer, uint32_t box_inner,
+                 uint32_t box_outer, int BK) {
+    const cuuint64_t dims[2] = {inner, outer};
+    const cuuint64_t strides[1] = {inner * 2};
+    const cuuint32_t box[2] = {box_inner, box_outer};
+    return tc_encode_tiled(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ptr, dims, strides, box,
+                           BK == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B);
 }
 
 bool tc_supported(int device) {
