@@ -676,6 +676,8 @@ inline int grid_axis(long long elements) { return grid_for((elements + axis_run(
 }  // namespace
 }  // namespace qn
 
+#include "qn_net_train.cuh"
+
 using namespace qn;
 
 struct qn_net {
@@ -853,6 +855,34 @@ static long long off_W(qn_net *n, int l) {
 static long long off_b(qn_net *n, int l) { return off_W(n, l) + (long long)n->C * n->C; }
 static long long off_wp(qn_net *n) { return block_base(n, n->L); }
 
+// Forward (and, with a target, loss and backward) through the fused kernels of
+// qn_net_train.cuh: 2 to 8 modes per axis. f, target: the caller's arrays, read in place.
+constexpr int kTrainMaxModes = 8;
+static bool net_fused(const qn_net *n) { return n->M >= 2 && n->M <= kTrainMaxModes; }
+
+static int net_fused_pass(qn_net *n, const float *f, const float *target, float *out, int B, cudaStream_t s) {
+    long long oR[16], oW[16], ob[16];
+    for (int l = 0; l < n->L; ++l) {
+        oR[l] = off_R(n, l);
+        oW[l] = off_W(n, l);
+        ob[l] = off_b(n, l);
+    }
+    TrNet t{n->G, n->M, n->L, B, f, target, n->basis_s, n->params, n->grads, n->t2, n->g, n->dhh, out, n->dout, n->dh,
+            n->loss, n->h.data(), n->z.data(), n->hh.data(), oR, oW, ob, off_wp(n)};
+    if (target != nullptr) {
+        QN_CUDA(cudaMemsetAsync(n->grads, 0, sizeof(float) * n->nparams, s));
+        QN_CUDA(cudaMemsetAsync(n->loss, 0, sizeof(double), s));
+    }
+    switch ((n->M + 1) / 2) {
+        case 1: tr_forward<2>(t, s); if (target) tr_backward<2>(t, s); break;
+        case 2: tr_forward<4>(t, s); if (target) tr_backward<4>(t, s); break;
+        case 3: tr_forward<6>(t, s); if (target) tr_backward<6>(t, s); break;
+        default: tr_forward<8>(t, s); if (target) tr_backward<8>(t, s); break;
+    }
+    QN_CUDA(cudaGetLastError());
+    return QN_OK;
+}
+
 // Forward pass on the coarse input already in n->fin (B samples); out in n->out.
 static int net_forward(qn_net *n, int B, cudaStream_t s) {
     const int G = n->G, C = n->C, M = n->M;
@@ -976,6 +1006,7 @@ extern "C" int qn_net_forward(qn_net *n, const float *f_coarse, float *out, int 
         return QN_EINVAL;
     }
     cudaStream_t s = (cudaStream_t)stream;
+    if (net_fused(n)) return net_fused_pass(n, f_coarse, nullptr, out, B, s);
     const long long pts = (long long)B * n->G * n->G * n->G;
     QN_CUDA(cudaMemcpyAsync(n->fin, f_coarse, sizeof(float) * pts, cudaMemcpyDeviceToDevice, s));
     rc = net_forward(n, B, s);
@@ -993,15 +1024,20 @@ extern "C" int qn_net_gradients(qn_net *n, const float *f_coarse, const float *t
         return QN_EINVAL;
     }
     cudaStream_t s = (cudaStream_t)stream;
-    const long long pts = (long long)B * n->G * n->G * n->G;
-    QN_CUDA(cudaMemcpyAsync(n->fin, f_coarse, sizeof(float) * pts, cudaMemcpyDeviceToDevice, s));
-    QN_CUDA(cudaMemcpyAsync(n->tgt, target, sizeof(float) * pts, cudaMemcpyDeviceToDevice, s));
-    rc = net_forward(n, B, s);
-    if (rc) return rc;
-    QN_CUDA(cudaMemsetAsync(n->loss, 0, sizeof(double), s));
-    k_mse<<<grid_for(pts), 256, 0, s>>>(n->out, n->tgt, n->dout, n->loss, pts);
-    rc = net_backward(n, B, s);
-    if (rc) return rc;
+    if (net_fused(n)) {
+        rc = net_fused_pass(n, f_coarse, target, n->out, B, s);
+        if (rc) return rc;
+    } else {
+        const long long pts = (long long)B * n->G * n->G * n->G;
+        QN_CUDA(cudaMemcpyAsync(n->fin, f_coarse, sizeof(float) * pts, cudaMemcpyDeviceToDevice, s));
+        QN_CUDA(cudaMemcpyAsync(n->tgt, target, sizeof(float) * pts, cudaMemcpyDeviceToDevice, s));
+        rc = net_forward(n, B, s);
+        if (rc) return rc;
+        QN_CUDA(cudaMemsetAsync(n->loss, 0, sizeof(double), s));
+        k_mse<<<grid_for(pts), 256, 0, s>>>(n->out, n->tgt, n->dout, n->loss, pts);
+        rc = net_backward(n, B, s);
+        if (rc) return rc;
+    }
     if (grads_out) QN_CUDA(cudaMemcpyAsync(grads_out, n->grads, sizeof(float) * n->nparams, cudaMemcpyDeviceToDevice, s));
     if (loss) {
         QN_CUDA(cudaMemcpyAsync(loss, n->loss, sizeof(double), cudaMemcpyDeviceToHost, s));

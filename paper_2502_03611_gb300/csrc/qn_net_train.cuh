@@ -1,0 +1,790 @@
+// Training kernels of the warm-start network (forward, loss, backward) for up to eight modes per
+// axis. Included by qn_net.cu.
+//
+// A block's work is bound by HBM once nothing is read twice: an activation of 8 x 64^3 nodes is
+// 134 MB in BF16 and a gradient 268 MB in FP32. Per block l the kernels are
+//   k_tr_analysis   one read of h_l (or of dh and z_l): the x and y analysis of a z plane per
+//                   CTA, which writes M^2 x 32 sums a plane instead of the x-analysed tensor;
+//   k_tr_mix        z analysis and channel mixing, one CTA per mode (backward: both gradients);
+//   k_tr_fwd        z_l = synthesis(g) + h_l W + b and h_{l+1}; the spectral term is formed in
+//                   registers per row. The last block also projects, takes the loss and its
+//                   gradient, and sums the projection's gradients;
+//   k_tr_bwd        dz = dh gelu'(z) again from dh and z (cheaper than storing dz), dW, db and
+//                   dh_prev = dz W^T + synthesis(dhh), in place of dh.
+// The lifted input h_0 = f wl + bl is formed where it is read (4 instead of 64 bytes a node), as
+// are the last block's dh = dout wp; block 0's dh_prev goes straight into the lift's gradients.
+//
+// The 32 x 32 channel products run on the tensor cores (mma.sync: register operands, 16 nodes of
+// one row per warp step) without losing FP32: a BF16 activation is one operand level, an FP32
+// operand three (x = x0 + x1 + x2, 24 bits), and the products down to 2^-24 of the leading one are
+// kept (3 for h W and h^T dz, 6 for dz W^T). Sums over nodes are added outside the tensor core,
+// in FP32 with rounding to nearest. Lanes own eight channels (8t .. 8t+7, t = lane & 3) of rows
+// g and g + 8 (g = lane >> 2): a permutation of the MMA's k and n indices that makes every load
+// and store 16 bytes wide.
+//
+// 10.4 -> 2.1 ms per loss + gradient at 64^3, batch 8.
+#pragma once
+
+#include <cuda_bf16.h>
+
+namespace qn {
+namespace {
+
+constexpr int kTrRows = 16;   // rows of one z plane per work item
+
+// gelu(x) = x sigmoid(2u), u = sqrt(2/pi) (x + 0.044715 x^3): the tanh form rewritten, without the
+// cancellation of 1 + tanh(u) at negative x.
+__device__ __forceinline__ float tr_gelu(float x) {
+    const float u2 = 2.0f * kGeluC * fmaf(0.044715f * x * x, x, x);
+    return x * __fdividef(1.0f, 1.0f + __expf(-u2));
+}
+
+// its derivative s + 2 x s (1 - s) u', s = sigmoid(2u), s (1 - s) = e s^2 with e = exp(-2u)
+__device__ __forceinline__ float tr_gelu_grad(float x) {
+    const float x2 = x * x;
+    const float u2 = 2.0f * kGeluC * fmaf(0.044715f * x2, x, x);
+    const float e = __expf(fminf(-u2, 80.0f));
+    const float s = __fdividef(1.0f, 1.0f + e);
+    return fmaf(2.0f * x * (e * s * s), kGeluC * fmaf(3.0f * 0.044715f, x2, 1.0f), s);
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&v);
+}
+__device__ __forceinline__ float bf_lo(uint32_t v) { return __uint_as_float(v << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
+
+// The next BF16 level of a pair; the arguments keep what it leaves.
+__device__ __forceinline__ uint32_t take_level(float &a, float &b) {
+    const uint32_t v = pack_bf16(a, b);
+    a -= bf_lo(v);
+    b -= bf_hi(v);
+    return v;
+}
+
+__device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                         uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ uint32_t trans8x8(uint32_t v) {
+    uint32_t r;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(v));
+    return r;
+}
+
+// Eight channels 8t .. 8t+7 of one node of the block's input: stored BF16, or lifted from f.
+template <bool LIFT>
+struct LoadH {
+    const __nv_bfloat16 *h;
+    const float *f;
+    float wl[8], bl[8];
+    __device__ __forceinline__ LoadH(const __nv_bfloat16 *h_, const float *f_, const float *wl_, const float *bl_, int t)
+        : h(h_ + (LIFT ? 0 : 8 * t)), f(f_) {
+        if (LIFT)
+            for (int j = 0; j < 8; ++j) {
+                wl[j] = wl_[8 * t + j];
+                bl[j] = bl_[8 * t + j];
+            }
+    }
+    __device__ __forceinline__ uint4 operator()(long long p, bool ok) const {
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (!ok) return v;
+        if (!LIFT) return *reinterpret_cast<const uint4 *>(h + p * 32);
+        const float x = f[p];
+        v.x = pack_bf16(fmaf(x, wl[0], bl[0]), fmaf(x, wl[1], bl[1]));
+        v.y = pack_bf16(fmaf(x, wl[2], bl[2]), fmaf(x, wl[3], bl[3]));
+        v.z = pack_bf16(fmaf(x, wl[4], bl[4]), fmaf(x, wl[5], bl[5]));
+        v.w = pack_bf16(fmaf(x, wl[6], bl[6]), fmaf(x, wl[7], bl[7]));
+        return v;
+    }
+};
+
+// What the analysis reads: the block's input (stored, or lifted from f), or dz in backward
+// (dh gelu'(z), or the last block's dout wp).
+enum TrSrc : int { TR_H = 0, TR_LIFT = 1, TR_DZ = 2, TR_DOUT = 3 };
+
+struct TrIn {
+    const __nv_bfloat16 *h, *z;
+    const float *f, *wl, *bl;   // lift
+    const float *dh;            // gradient of the block's output, or dout (TR_DOUT)
+    const float *wp;
+};
+
+template <int SRC>
+struct LoadV {
+    LoadH<SRC == TR_LIFT> lh;
+    const TrIn in;
+    float wp[8];
+    int t;
+    __device__ __forceinline__ LoadV(const TrIn &i, int t_) : lh(i.h, i.f, i.wl, i.bl, t_), in(i), t(t_) {
+        if (SRC == TR_DOUT)
+            for (int j = 0; j < 8; ++j) wp[j] = i.wp[8 * t_ + j];
+    }
+    __device__ __forceinline__ void operator()(long long p, bool ok, float (&v)[8]) const {
+        if (SRC == TR_H || SRC == TR_LIFT) {
+            const uint4 o = lh(p, ok);
+            const uint32_t w[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                v[2 * j] = bf_lo(w[j]);
+                v[2 * j + 1] = bf_hi(w[j]);
+            }
+        } else if (SRC == TR_DOUT) {
+            const float d = ok ? in.dh[p] : 0.0f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = d * wp[j];
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = 0.0f;
+            if (!ok) return;
+            const float4 d0 = *reinterpret_cast<const float4 *>(in.dh + p * 32 + 8 * t);
+            const float4 d1 = *reinterpret_cast<const float4 *>(in.dh + p * 32 + 8 * t + 4);
+            const uint4 o = *reinterpret_cast<const uint4 *>(in.z + p * 32 + 8 * t);
+            v[0] = d0.x * tr_gelu_grad(bf_lo(o.x));
+            v[1] = d0.y * tr_gelu_grad(bf_hi(o.x));
+            v[2] = d0.z * tr_gelu_grad(bf_lo(o.y));
+            v[3] = d0.w * tr_gelu_grad(bf_hi(o.y));
+            v[4] = d1.x * tr_gelu_grad(bf_lo(o.z));
+            v[5] = d1.y * tr_gelu_grad(bf_hi(o.z));
+            v[6] = d1.z * tr_gelu_grad(bf_lo(o.w));
+            v[7] = d1.w * tr_gelu_grad(bf_hi(o.w));
+        }
+    }
+};
+
+// t2[plane][ky][kx][c] = sum_y sum_x B[y][ky] B[x][kx] v[plane][y][x][c], one CTA per plane
+// (b, z). basis: [G][M]; MP = M rounded up to even (the extra mode is zero).
+template <int MP, int SRC>
+__global__ void __launch_bounds__(256, 2) k_tr_analysis(const TrIn in, const float *__restrict__ basis, int G, int M,
+                                                        float *__restrict__ t2) {
+    __shared__ float sB[256 * MP];
+    __shared__ float sQ[MP * MP * 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    for (int e = threadIdx.x; e < MP * G; e += 256) {
+        const int x = e / MP, k = e % MP;
+        sB[e] = (k < M) ? basis[x * M + k] : 0.0f;
+    }
+    for (int e = threadIdx.x; e < MP * MP * 32; e += 256) sQ[e] = 0.0f;
+    __syncthreads();
+    const LoadV<SRC> load(in, t);
+    float Q[MP][MP];
+#pragma unroll
+    for (int a = 0; a < MP; ++a)
+#pragma unroll
+        for (int k = 0; k < MP; ++k) Q[a][k] = 0.0f;
+    for (int y = warp; y < G; y += 8) {
+        const long long row = ((long long)blockIdx.x * G + y) * G;
+        float acc[MP][8];
+#pragma unroll
+        for (int k = 0; k < MP; ++k)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[k][j] = 0.0f;
+#pragma unroll 4
+        for (int x0 = 0; x0 < G; x0 += 8) {
+            const int x = x0 + g;
+            float v[8];
+            load(row + x, x < G, v);
+            const float *b = sB + min(x, G - 1) * MP;
+#pragma unroll
+            for (int k = 0; k < MP; ++k)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[k][j] = fmaf(b[k], v[j], acc[k][j]);
+        }
+        // sum over the eight g lanes, halving the channels a lane holds each time
+        const bool u2 = lane & 16, u1 = lane & 8, u0 = lane & 4;
+        float T[MP];
+#pragma unroll
+        for (int k = 0; k < MP; ++k) {
+            float r4[4], r2[2];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                r4[j] = (u2 ? acc[k][j + 4] : acc[k][j]) + __shfl_xor_sync(0xffffffffu, u2 ? acc[k][j] : acc[k][j + 4], 16);
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                r2[j] = (u1 ? r4[j + 2] : r4[j]) + __shfl_xor_sync(0xffffffffu, u1 ? r4[j] : r4[j + 2], 8);
+            T[k] = (u0 ? r2[1] : r2[0]) + __shfl_xor_sync(0xffffffffu, u0 ? r2[0] : r2[1], 4);
+        }
+#pragma unroll
+        for (int a = 0; a < MP; ++a) {
+            const float b = sB[y * MP + a];
+#pragma unroll
+            for (int k = 0; k < MP; ++k) Q[a][k] = fmaf(b, T[k], Q[a][k]);
+        }
+    }
+    const int c = 8 * t + 4 * ((lane >> 4) & 1) + 2 * ((lane >> 3) & 1) + ((lane >> 2) & 1);   // this lane's channel
+    for (int w = 0; w < 8; ++w) {   // the warps' sums in a fixed order
+        if (warp == w)
+#pragma unroll
+            for (int a = 0; a < MP; ++a)
+#pragma unroll
+                for (int k = 0; k < MP; ++k) sQ[(a * MP + k) * 32 + c] += Q[a][k];
+        __syncthreads();
+    }
+    float *o = t2 + (long long)blockIdx.x * MP * MP * 32;
+    for (int e = threadIdx.x; e < MP * MP * 32; e += 256) o[e] = sQ[e];
+}
+
+// The z analysis of one mode k = (kz, ky, kx), all samples (one warp each): lane = channel.
+__device__ __forceinline__ float z_analysis(const float *__restrict__ t2, const float *__restrict__ basis, int b, int G,
+                                            int M, int MP, int k, int lane) {
+    const int kz = k / (M * M), ky = k / M % M, kx = k % M;
+    const float *p = t2 + ((long long)b * G * MP * MP + ky * MP + kx) * 32 + lane;
+    const int stride = MP * MP * 32;
+    float a0 = 0.0f, a1 = 0.0f;
+#pragma unroll 4
+    for (int z = 0; z + 1 < G; z += 2) {
+        a0 = fmaf(__ldg(basis + z * M + kz), __ldg(p + (long long)z * stride), a0);
+        a1 = fmaf(__ldg(basis + (z + 1) * M + kz), __ldg(p + (long long)(z + 1) * stride), a1);
+    }
+    if (G & 1) a0 = fmaf(__ldg(basis + (G - 1) * M + kz), __ldg(p + (long long)(G - 1) * stride), a0);
+    return a0 + a1;
+}
+
+// hh[b][k][c], g[b][k][o] = sum_i hh[b][k][i] R[k][i][o]; one CTA per mode.
+__global__ void __launch_bounds__(256) k_tr_mix(const float *__restrict__ t2, const float *__restrict__ basis, int B,
+                                                int G, int M, int MP, const float *__restrict__ R,
+                                                float *__restrict__ hh, float *__restrict__ g) {
+    const int lane = threadIdx.x & 31, k = blockIdx.x, K = gridDim.x;
+    for (int b = threadIdx.x >> 5; b < B; b += 8) {
+        const float v = z_analysis(t2, basis, b, G, M, MP, k, lane);
+        hh[((long long)b * K + k) * 32 + lane] = v;
+        float s = 0.0f;
+#pragma unroll 8
+        for (int i = 0; i < 32; ++i)
+            s = fmaf(__shfl_sync(0xffffffffu, v, i), __ldg(R + (long long)k * 1024 + i * 32 + lane), s);
+        g[((long long)b * K + k) * 32 + lane] = s;
+    }
+}
+
+// dg = z analysis of dz's sums; dhh[b][k][i] = sum_o dg[b][k][o] R[k][i][o]; dR[k][i][o] =
+// sum_b hh[b][k][i] dg[b][k][o] in order of b. One CTA per mode.
+__global__ void __launch_bounds__(256) k_tr_mix_bwd(const float *__restrict__ t2, const float *__restrict__ basis, int B,
+                                                    int G, int M, int MP, const float *__restrict__ R,
+                                                    const float *__restrict__ hh, float *__restrict__ dhh,
+                                                    float *__restrict__ dR) {
+    __shared__ float sR[32 * 33], sdg[64 * 32], shh[64 * 32];
+    const int lane = threadIdx.x & 31, k = blockIdx.x, K = gridDim.x;
+    for (int e = threadIdx.x; e < 1024; e += 256) sR[(e >> 5) * 33 + (e & 31)] = R[(long long)k * 1024 + e];
+    for (int b = threadIdx.x >> 5; b < B; b += 8) {
+        sdg[b * 32 + lane] = z_analysis(t2, basis, b, G, M, MP, k, lane);
+        shh[b * 32 + lane] = hh[((long long)b * K + k) * 32 + lane];
+    }
+    __syncthreads();
+    for (int b = threadIdx.x >> 5; b < B; b += 8) {
+        float s = 0.0f;
+#pragma unroll 8
+        for (int o = 0; o < 32; ++o) s = fmaf(sdg[b * 32 + o], sR[lane * 33 + o], s);
+        dhh[((long long)b * K + k) * 32 + lane] = s;
+    }
+    for (int e = threadIdx.x; e < 1024; e += 256) {
+        float s = 0.0f;
+        for (int b = 0; b < B; ++b) s = fmaf(shh[b * 32 + (e >> 5)], sdg[b * 32 + (e & 31)], s);
+        dR[(long long)k * 1024 + e] = s;
+    }
+}
+
+// MMA fragments of a 32 x 32 matrix X[k][n] in three BF16 levels, k and n permuted as the lanes
+// own channels: sW[level][k half][n pair][lane] holds the B operands of two column tiles.
+__device__ __forceinline__ void load_fragments(uint4 *sW, const float *X, bool transpose, int threads) {
+    for (int e = threadIdx.x; e < 2 * 2 * 32; e += threads) {
+        const int lane = e & 31, np = (e >> 5) & 1, ks = e >> 6;
+        const int g = lane >> 2, t = lane & 3;
+        uint32_t lv[3][4];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int n = 8 * (g >> 1) + 2 * (2 * np + q) + (g & 1);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int k = 8 * t + 4 * ks + 2 * h;
+                float a = transpose ? X[n * 32 + k] : X[k * 32 + n];
+                float b = transpose ? X[n * 32 + k + 1] : X[(k + 1) * 32 + n];
+#pragma unroll
+                for (int l = 0; l < 3; ++l) lv[l][2 * q + h] = take_level(a, b);
+            }
+        }
+#pragma unroll
+        for (int l = 0; l < 3; ++l)
+            sW[((l * 2 + ks) * 2 + np) * 32 + lane] = make_uint4(lv[l][0], lv[l][1], lv[l][2], lv[l][3]);
+    }
+}
+
+// sS[ky][kx][c] = sum_kz B[z][kz] g[b][kz][ky][kx][c] of one plane.
+template <int MP>
+__device__ __forceinline__ void z_synthesis(float *sS, const float *sB, const float *__restrict__ g, int b, int z, int M,
+                                            int threads) {
+    const float *gb = g + (long long)b * M * M * M * 32;
+    for (int e = threadIdx.x; e < MP * MP * 32; e += threads) {
+        const int kk = e >> 5, ky = kk / MP, kx = kk % MP;
+        float a = 0.0f;
+        if (ky < M && kx < M)
+            for (int k = 0; k < M; ++k) a = fmaf(sB[z * MP + k], __ldg(gb + ((k * M + ky) * M + kx) * 32 + (e & 31)), a);
+        sS[e] = a;
+    }
+}
+
+// sT[kx][c] = sum_ky B[y][ky] sS[ky][kx][c] of one row, by one warp (lane = channel).
+template <int MP>
+__device__ __forceinline__ void y_synthesis(float *sT, const float *sS, const float *sB, int y, int lane) {
+    __syncwarp();
+#pragma unroll
+    for (int kx = 0; kx < MP; ++kx) {
+        float a = 0.0f;
+#pragma unroll
+        for (int ky = 0; ky < MP; ++ky) a = fmaf(sB[y * MP + ky], sS[(ky * MP + kx) * 32 + lane], a);
+        sT[kx * 32 + lane] = a;
+    }
+    __syncwarp();
+}
+
+struct TrFwd {
+    TrIn in;
+    const float *basis, *g, *W, *bvec;
+    __nv_bfloat16 *z, *hnext;
+    int B, G, M;
+    // last block: projection, and with a target the loss and its gradients
+    const float *wp, *bp, *target;
+    float *out, *dout, *dwp, *dbp;
+    double *loss;
+};
+
+template <int MP, bool LIFT, bool LAST>
+__global__ void __launch_bounds__(256, 2) k_tr_fwd(const TrFwd a) {
+    __shared__ float sB[256 * MP];
+    __shared__ __align__(16) float sS[MP * MP * 32];
+    __shared__ __align__(16) float sT[8][MP * 32];
+    __shared__ uint4 sW[3 * 2 * 2 * 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const int G = a.G, M = a.M;
+    for (int e = threadIdx.x; e < MP * G; e += 256) {
+        const int x = e / MP, k = e % MP;
+        sB[e] = (k < M) ? a.basis[x * M + k] : 0.0f;
+    }
+    load_fragments(sW, a.W, false, 256);
+    const LoadH<LIFT> load(a.in.h, a.in.f, a.in.wl, a.in.bl, t);
+    float bias[8], wp[LAST ? 8 : 1], gw[LAST ? 8 : 1], gb = 0.0f, bp = 0.0f, inv = 0.0f;
+    double loss = 0.0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) bias[j] = a.bvec[8 * t + j];
+    if constexpr (LAST) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            wp[j] = a.wp[8 * t + j];
+            gw[j] = 0.0f;
+        }
+        bp = a.bp[0];
+        inv = 1.0f / (float)((long long)a.B * G * G * G);
+    }
+    const int chunks = (G + kTrRows - 1) / kTrRows;
+    const int items = a.B * G * chunks;
+    for (int it = blockIdx.x; it < items; it += gridDim.x) {
+        const int plane = it / chunks, y0 = (it % chunks) * kTrRows, y1 = min(y0 + kTrRows, G);
+        __syncthreads();
+        z_synthesis<MP>(sS, sB, a.g, plane / G, plane % G, M, 256);
+        __syncthreads();
+        for (int y = y0 + warp; y < y1; y += 8) {
+            y_synthesis<MP>(sT[warp], sS, sB, y, lane);
+            float T[MP][8];
+#pragma unroll
+            for (int k = 0; k < MP; ++k) {
+                const float4 u = *reinterpret_cast<const float4 *>(sT[warp] + k * 32 + 8 * t);
+                const float4 v = *reinterpret_cast<const float4 *>(sT[warp] + k * 32 + 8 * t + 4);
+                T[k][0] = u.x, T[k][1] = u.y, T[k][2] = u.z, T[k][3] = u.w;
+                T[k][4] = v.x, T[k][5] = v.y, T[k][6] = v.z, T[k][7] = v.w;
+            }
+            const long long row = ((long long)plane * G + y) * G;
+            uint4 hA = load(row + g, g < G), hB = load(row + 8 + g, 8 + g < G);
+            for (int x0 = 0; x0 < G; x0 += 16) {
+                const uint4 cA = hA, cB = hB;
+                const int xn = x0 + 16 + g;
+                hA = load(row + xn, xn < G);
+                hB = load(row + xn + 8, xn + 8 < G);
+                float d[4][4];
+#pragma unroll
+                for (int n = 0; n < 4; ++n) d[n][0] = d[n][1] = d[n][2] = d[n][3] = 0.0f;
+#pragma unroll
+                for (int l = 2; l >= 0; --l)
+#pragma unroll
+                    for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+                        for (int np = 0; np < 2; ++np) {
+                            const uint4 w = sW[((l * 2 + ks) * 2 + np) * 32 + lane];
+                            const uint32_t a0 = ks ? cA.z : cA.x, a1 = ks ? cB.z : cB.x;
+                            const uint32_t a2 = ks ? cA.w : cA.y, a3 = ks ? cB.w : cB.y;
+                            mma16816(d[2 * np], a0, a1, a2, a3, w.x, w.y);
+                            mma16816(d[2 * np + 1], a0, a1, a2, a3, w.z, w.w);
+                        }
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const int x = x0 + 8 * r + g;
+                    const bool ok = x < G;
+                    float s[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) s[j] = bias[j];
+                    const float *b = sB + min(x, G - 1) * MP;
+#pragma unroll
+                    for (int k = 0; k < MP; ++k)
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) s[j] = fmaf(b[k], T[k][j], s[j]);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) s[j] += d[j >> 1][2 * r + (j & 1)];
+                    const long long p = row + x;
+                    uint4 o;
+                    if (LAST || a.z != nullptr) {
+                        o = make_uint4(pack_bf16(s[0], s[1]), pack_bf16(s[2], s[3]), pack_bf16(s[4], s[5]),
+                                       pack_bf16(s[6], s[7]));
+                        if (!LAST && ok) *reinterpret_cast<uint4 *>(a.z + p * 32 + 8 * t) = o;
+                    }
+                    if constexpr (!LAST) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) s[j] = tr_gelu(s[j]);
+                        o = make_uint4(pack_bf16(s[0], s[1]), pack_bf16(s[2], s[3]), pack_bf16(s[4], s[5]),
+                                       pack_bf16(s[6], s[7]));
+                        if (ok) *reinterpret_cast<uint4 *>(a.hnext + p * 32 + 8 * t) = o;
+                    } else {
+                        const float hv[8] = {bf_lo(o.x), bf_hi(o.x), bf_lo(o.y), bf_hi(o.y),
+                                             bf_lo(o.z), bf_hi(o.z), bf_lo(o.w), bf_hi(o.w)};
+                        float v = 0.0f;
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) v = fmaf(hv[j], wp[j], v);
+                        v += __shfl_xor_sync(0xffffffffu, v, 1);
+                        v += __shfl_xor_sync(0xffffffffu, v, 2);
+                        v += bp;
+                        if (ok) {   // h_L itself is not stored: nothing reads it
+                            if (t == 0) a.out[p] = v;
+                            if (a.target != nullptr) {
+                                const float e = v - a.target[p];
+                                const float dd = 2.0f * e * inv;
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) gw[j] = fmaf(dd, hv[j], gw[j]);
+                                if (t == 0) {
+                                    a.dout[p] = dd;
+                                    gb += dd;
+                                    loss += (double)e * e;
+                                }
+                            }
+                        }
+                    }
+                }
+            }
+        }
+    }
+    if constexpr (LAST) {
+        if (a.target == nullptr) return;
+        // the projection's gradients and the loss: lanes of one t, then the warps
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) gw[j] += __shfl_xor_sync(0xffffffffu, gw[j], o);
+            gb += __shfl_xor_sync(0xffffffffu, gb, o);
+            loss += __shfl_xor_sync(0xffffffffu, loss, o);
+        }
+        __syncthreads();
+        if (g == 0)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) sT[warp][8 * t + j] = gw[j];
+        if (lane == 0) {
+            sT[warp][32] = gb;
+            atomicAdd(a.loss, loss / (double)((long long)a.B * G * G * G));
+        }
+        __syncthreads();
+        if (threadIdx.x < 33) {
+            float s = 0.0f;
+            for (int w = 0; w < 8; ++w) s += sT[w][threadIdx.x];
+            atomicAdd(threadIdx.x < 32 ? a.dwp + threadIdx.x : a.dbp, s);
+        }
+    }
+}
+
+struct TrBwd {
+    TrIn in;
+    const float *basis, *dhh, *W;
+    float *dh_prev;             // block 0: not written, goes into dwl, dbl
+    float *dW, *db, *dwl, *dbl;
+    int B, G, M;
+};
+
+template <int MP, bool FIRST, bool LAST>
+__global__ void __launch_bounds__(128, 3) k_tr_bwd(const TrBwd a) {
+    __shared__ float sB[256 * MP];
+    __shared__ __align__(16) float sS[MP * MP * 32 < 1024 + 96 ? 1024 + 96 : MP * MP * 32];
+    __shared__ __align__(16) float sT[4][MP * 32];
+    __shared__ uint4 sW[3 * 2 * 2 * 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const int G = a.G, M = a.M;
+    for (int e = threadIdx.x; e < MP * G; e += 128) {
+        const int x = e / MP, k = e % MP;
+        sB[e] = (k < M) ? a.basis[x * M + k] : 0.0f;
+    }
+    load_fragments(sW, a.W, true, 128);
+    const LoadH<FIRST> load_h(a.in.h, a.in.f, a.in.wl, a.in.bl, t);
+    const LoadV<LAST ? TR_DOUT : TR_DZ> load_dz(a.in, t);
+    float dW[2][4][4], db[8], gl[FIRST ? 8 : 1], gbl[FIRST ? 8 : 1];
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int n = 0; n < 4; ++n) dW[m][n][0] = dW[m][n][1] = dW[m][n][2] = dW[m][n][3] = 0.0f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        db[j] = 0.0f;
+        if constexpr (FIRST) gl[j] = gbl[j] = 0.0f;
+    }
+    const int chunks = (G + kTrRows - 1) / kTrRows;
+    const int items = a.B * G * chunks;
+    for (int it = blockIdx.x; it < items; it += gridDim.x) {
+        const int plane = it / chunks, y0 = (it % chunks) * kTrRows, y1 = min(y0 + kTrRows, G);
+        __syncthreads();
+        z_synthesis<MP>(sS, sB, a.dhh, plane / G, plane % G, M, 128);
+        __syncthreads();
+        for (int y = y0 + warp; y < y1; y += 4) {
+            y_synthesis<MP>(sT[warp], sS, sB, y, lane);
+            const long long row = ((long long)plane * G + y) * G;
+            for (int x0 = 0; x0 < G; x0 += 16) {
+                const int xA = x0 + g, xB = x0 + 8 + g;
+                float vA[8], vB[8];
+                load_dz(row + xA, xA < G, vA);
+                load_dz(row + xB, xB < G, vB);
+                const uint4 oA = load_h(row + xA, xA < G), oB = load_h(row + xB, xB < G);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) db[j] += vA[j] + vB[j];
+                uint32_t lA[3][4], lB[3][4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int l = 0; l < 3; ++l) {
+                        lA[l][j] = take_level(vA[2 * j], vA[2 * j + 1]);
+                        lB[l][j] = take_level(vB[2 * j], vB[2 * j + 1]);
+                    }
+                // dW += h^T dz over the 16 nodes
+                {
+                    const uint32_t hA[4] = {oA.x, oA.y, oA.z, oA.w}, hB[4] = {oB.x, oB.y, oB.z, oB.w};
+                    uint32_t tA[4], tB[4];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        tA[r] = trans8x8(hA[r]);
+                        tB[r] = trans8x8(hB[r]);
+                    }
+#pragma unroll
+                    for (int n = 0; n < 4; ++n) {
+                        float d[2][4] = {{0.0f, 0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f, 0.0f}};
+#pragma unroll
+                        for (int l = 2; l >= 0; --l) {
+                            const uint32_t b0 = trans8x8(lA[l][n]), b1 = trans8x8(lB[l][n]);
+#pragma unroll
+                            for (int m = 0; m < 2; ++m)
+                                mma16816(d[m], tA[2 * m], tA[2 * m + 1], tB[2 * m], tB[2 * m + 1], b0, b1);
+                        }
+#pragma unroll
+                        for (int m = 0; m < 2; ++m)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) dW[m][n][e] += d[m][e];
+                    }
+                }
+                // dh_prev = dz W^T + synthesis
+                float d[4][4];
+#pragma unroll
+                for (int n = 0; n < 4; ++n) d[n][0] = d[n][1] = d[n][2] = d[n][3] = 0.0f;
+#pragma unroll
+                for (int lw = 2; lw >= 0; --lw)
+#pragma unroll
+                    for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+                        for (int np = 0; np < 2; ++np) {
+                            const uint4 w = sW[((lw * 2 + ks) * 2 + np) * 32 + lane];
+#pragma unroll
+                            for (int l = 2; l >= 0; --l) {
+                                if (l + lw > 2) continue;
+                                mma16816(d[2 * np], lA[l][2 * ks], lB[l][2 * ks], lA[l][2 * ks + 1], lB[l][2 * ks + 1],
+                                         w.x, w.y);
+                                mma16816(d[2 * np + 1], lA[l][2 * ks], lB[l][2 * ks], lA[l][2 * ks + 1],
+                                         lB[l][2 * ks + 1], w.z, w.w);
+                            }
+                        }
+                float s[2][8];
+                const float *bA = sB + min(xA, G - 1) * MP, *bB = sB + min(xB, G - 1) * MP;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) s[0][j] = s[1][j] = 0.0f;
+#pragma unroll
+                for (int k = 0; k < MP; ++k) {
+                    const float4 u = *reinterpret_cast<const float4 *>(sT[warp] + k * 32 + 8 * t);
+                    const float4 v = *reinterpret_cast<const float4 *>(sT[warp] + k * 32 + 8 * t + 4);
+                    const float T[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        s[0][j] = fmaf(bA[k], T[j], s[0][j]);
+                        s[1][j] = fmaf(bB[k], T[j], s[1][j]);
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const int x = x0 + 8 * r + g;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) s[r][j] += d[j >> 1][2 * r + (j & 1)];
+                    if (x >= G) continue;
+                    if constexpr (FIRST) {
+                        const float fv = a.in.f[row + x];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            gl[j] = fmaf(fv, s[r][j], gl[j]);
+                            gbl[j] += s[r][j];
+                        }
+                    } else {
+                        float4 *o = reinterpret_cast<float4 *>(a.dh_prev + (row + x) * 32 + 8 * t);
+                        o[0] = make_float4(s[r][0], s[r][1], s[r][2], s[r][3]);
+                        o[1] = make_float4(s[r][4], s[r][5], s[r][6], s[r][7]);
+                    }
+                }
+            }
+        }
+    }
+    // sums over the lanes of one t, then over the warps in a fixed order, then one atomic each
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+            db[j] += __shfl_xor_sync(0xffffffffu, db[j], o);
+            if constexpr (FIRST) {
+                gl[j] += __shfl_xor_sync(0xffffffffu, gl[j], o);
+                gbl[j] += __shfl_xor_sync(0xffffffffu, gbl[j], o);
+            }
+        }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 1024 + 96; e += 128) sS[e] = 0.0f;
+    __syncthreads();
+    for (int w = 0; w < 4; ++w) {
+        if (warp == w) {
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int n = 0; n < 4; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int i = 8 * (g >> 1) + 2 * (2 * m + (e >> 1)) + (g & 1), o = 8 * t + 2 * n + (e & 1);
+                        sS[i * 32 + o] += dW[m][n][e];
+                    }
+            if (g == 0)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    sS[1024 + 8 * t + j] += db[j];
+                    if constexpr (FIRST) {
+                        sS[1056 + 8 * t + j] += gl[j];
+                        sS[1088 + 8 * t + j] += gbl[j];
+                    }
+                }
+        }
+        __syncthreads();
+    }
+    for (int e = threadIdx.x; e < 1024 + (FIRST ? 96 : 32); e += 128) {
+        float *o = e < 1024 ? a.dW + e : (e < 1056 ? a.db + (e - 1024) : (e < 1088 ? a.dwl + (e - 1056) : a.dbl + (e - 1088)));
+        atomicAdd(o, sS[e]);
+    }
+}
+
+// Forward pass of B samples (f: [B][G^3]); with a target the loss, dout and the projection's
+// gradients too (the gradient array must be zero).
+struct TrNet {
+    int G, M, L, B;
+    const float *f, *target, *basis;
+    float *params, *grads, *t2, *g, *dhh, *out, *dout, *dh;
+    double *loss;
+    __nv_bfloat16 *const *h, *const *z;
+    float *const *hh;
+    const long long *off_R, *off_W, *off_b;
+    long long off_wp;
+};
+
+template <int MP>
+void tr_forward(const TrNet &n, cudaStream_t s) {
+    const int planes = n.B * n.G, K = n.M * n.M * n.M;
+    const int items = planes * ((n.G + kTrRows - 1) / kTrRows);
+    const int grid = items < 2 * 152 ? items : 2 * 152;
+    for (int l = 0; l < n.L; ++l) {
+        TrFwd a{};
+        a.in.h = n.h[l];
+        a.in.f = n.f;
+        a.in.wl = n.params;
+        a.in.bl = n.params + 32;
+        if (l == 0)
+            k_tr_analysis<MP, TR_LIFT><<<planes, 256, 0, s>>>(a.in, n.basis, n.G, n.M, n.t2);
+        else
+            k_tr_analysis<MP, TR_H><<<planes, 256, 0, s>>>(a.in, n.basis, n.G, n.M, n.t2);
+        k_tr_mix<<<K, 256, 0, s>>>(n.t2, n.basis, n.B, n.G, n.M, MP, n.params + n.off_R[l], n.hh[l], n.g);
+        a.basis = n.basis;
+        a.g = n.g;
+        a.W = n.params + n.off_W[l];
+        a.bvec = n.params + n.off_b[l];
+        a.z = n.target != nullptr ? n.z[l] : nullptr;
+        a.hnext = n.h[l + 1];
+        a.B = n.B;
+        a.G = n.G;
+        a.M = n.M;
+        a.wp = n.params + n.off_wp;
+        a.bp = a.wp + 32;
+        a.target = n.target;
+        a.out = n.out;
+        a.dout = n.dout;
+        a.dwp = n.grads + n.off_wp;
+        a.dbp = a.dwp + 32;
+        a.loss = n.loss;
+        const bool last = l == n.L - 1;
+        if (l == 0 && last)
+            k_tr_fwd<MP, true, true><<<grid, 256, 0, s>>>(a);
+        else if (l == 0)
+            k_tr_fwd<MP, true, false><<<grid, 256, 0, s>>>(a);
+        else if (last)
+            k_tr_fwd<MP, false, true><<<grid, 256, 0, s>>>(a);
+        else
+            k_tr_fwd<MP, false, false><<<grid, 256, 0, s>>>(a);
+    }
+}
+
+template <int MP>
+void tr_backward(const TrNet &n, cudaStream_t s) {
+    const int planes = n.B * n.G, K = n.M * n.M * n.M;
+    const int items = planes * ((n.G + kTrRows - 1) / kTrRows);
+    const int grid = items < 3 * 152 ? items : 3 * 152;
+    for (int l = n.L - 1; l >= 0; --l) {
+        const bool last = l == n.L - 1;
+        TrBwd a{};
+        a.in.h = n.h[l];
+        a.in.z = n.z[l];
+        a.in.f = n.f;
+        a.in.wl = n.params;
+        a.in.bl = n.params + 32;
+        a.in.dh = last ? n.dout : n.dh;
+        a.in.wp = n.params + n.off_wp;
+        if (last)
+            k_tr_analysis<MP, TR_DOUT><<<planes, 256, 0, s>>>(a.in, n.basis, n.G, n.M, n.t2);
+        else
+            k_tr_analysis<MP, TR_DZ><<<planes, 256, 0, s>>>(a.in, n.basis, n.G, n.M, n.t2);
+        k_tr_mix_bwd<<<K, 256, 0, s>>>(n.t2, n.basis, n.B, n.G, n.M, MP, n.params + n.off_R[l], n.hh[l], n.dhh,
+                                       n.grads + n.off_R[l]);
+        a.basis = n.basis;
+        a.dhh = n.dhh;
+        a.W = n.params + n.off_W[l];
+        a.dh_prev = n.dh;
+        a.dW = n.grads + n.off_W[l];
+        a.db = n.grads + n.off_b[l];
+        a.dwl = n.grads;
+        a.dbl = n.grads + 32;
+        a.B = n.B;
+        a.G = n.G;
+        a.M = n.M;
+        if (l == 0 && last)
+            k_tr_bwd<MP, true, true><<<grid, 128, 0, s>>>(a);
+        else if (l == 0)
+            k_tr_bwd<MP, true, false><<<grid, 128, 0, s>>>(a);
+        else if (last)
+            k_tr_bwd<MP, false, true><<<grid, 128, 0, s>>>(a);
+        else
+            k_tr_bwd<MP, false, false><<<grid, 128, 0, s>>>(a);
+    }
+}
+
+}  // namespace
+}  // namespace qn
