@@ -788,7 +788,11 @@ extern "C" int qn_net_create(int G, int channels, int modes, int blocks, int max
         NCK(cudaMalloc(&n->z[l], sizeof(__nv_bfloat16) * act));
         NCK(cudaMalloc(&n->hh[l], sizeof(float) * max_batch * K * channels));
     }
-    const long long tsz = (long long)max_batch * G * G * modes * channels;
+    // x-analysed tensor (unfused kernels), or the fused kernels' sums per plane and part
+    const long long mp = (modes + 1) / 2 * 2;
+    long long tsz = (long long)max_batch * G * G * modes * channels;
+    if (tsz < (long long)max_batch * G * kTrParts * mp * mp * channels)
+        tsz = (long long)max_batch * G * kTrParts * mp * mp * channels;
     NCK(cudaMalloc(&n->t1, sizeof(float) * tsz));
     NCK(cudaMalloc(&n->t2, sizeof(float) * tsz));
     NCK(cudaMalloc(&n->sp, sizeof(float) * act));
@@ -807,6 +811,15 @@ extern "C" int qn_net_create(int G, int channels, int modes, int blocks, int max
         const long long chunks = (G + kInfRows - 1) / kInfRows;
         NCK(cudaMalloc(&n->part, sizeof(float) * (size_t)(G * chunks * modes * modes * channels)));
         NCK(cudaMalloc(&n->wsq, 2 * sizeof(double)));
+    }
+    if (modes >= 2 && modes <= 8) {
+        const int rc = modes <= 2 ? tr_set_attributes<2>()
+                                  : (modes <= 4 ? tr_set_attributes<4>()
+                                                : (modes <= 6 ? tr_set_attributes<6>() : tr_set_attributes<8>()));
+        if (rc != QN_OK) {
+            net_free(n);
+            return rc;
+        }
     }
     n->step = 0;
     *out = n;

@@ -78,35 +78,28 @@ __device__ __forceinline__ uint32_t trans8x8(uint32_t v) {
     return r;
 }
 
-// Eight channels 8t .. 8t+7 of one node of the block's input: stored BF16, or lifted from f.
-template <bool LIFT>
-struct LoadH {
-    const __nv_bfloat16 *h;
-    const float *f;
-    float wl[8], bl[8];
-    __device__ __forceinline__ LoadH(const __nv_bfloat16 *h_, const float *f_, const float *wl_, const float *bl_, int t)
-        : h(h_ + (LIFT ? 0 : 8 * t)), f(f_) {
-        if (LIFT)
-            for (int j = 0; j < 8; ++j) {
-                wl[j] = wl_[8 * t + j];
-                bl[j] = bl_[8 * t + j];
-            }
-    }
-    __device__ __forceinline__ uint4 operator()(long long p, bool ok) const {
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (!ok) return v;
-        if (!LIFT) return *reinterpret_cast<const uint4 *>(h + p * 32);
-        const float x = f[p];
-        v.x = pack_bf16(fmaf(x, wl[0], bl[0]), fmaf(x, wl[1], bl[1]));
-        v.y = pack_bf16(fmaf(x, wl[2], bl[2]), fmaf(x, wl[3], bl[3]));
-        v.z = pack_bf16(fmaf(x, wl[4], bl[4]), fmaf(x, wl[5], bl[5]));
-        v.w = pack_bf16(fmaf(x, wl[6], bl[6]), fmaf(x, wl[7], bl[7]));
-        return v;
-    }
-};
+// 16 or 4 bytes global -> shared without a register; `ok` false writes zeros.
+__device__ __forceinline__ void copy16(void *dst, const void *src, bool ok) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(ok ? 16 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void copy4(void *dst, const void *src, bool ok) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(ok ? 4 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 
-// What the analysis reads: the block's input (stored, or lifted from f), or dz in backward
-// (dh gelu'(z), or the last block's dout wp).
+// What a step of eight nodes reads, eight channels a lane: the block's input (stored BF16, or
+// lifted from f), or dz in backward (dh gelu'(z), or the last block's dout wp). One lane's
+// pieces go through its own slots of a shared-memory ring (it alone writes and reads them, so no
+// barrier is needed), a fixed number of steps ahead: the loads of a register pipeline that deep
+// would not fit, and with one step in flight these kernels waited on memory most of the time.
 enum TrSrc : int { TR_H = 0, TR_LIFT = 1, TR_DZ = 2, TR_DOUT = 3 };
 
 struct TrIn {
@@ -116,95 +109,161 @@ struct TrIn {
     const float *wp;
 };
 
+// 16-byte pieces of one lane and one step in the ring
+__host__ __device__ constexpr int tr_pieces(int src) { return src == TR_DZ ? 3 : 1; }
+
 template <int SRC>
-struct LoadV {
-    LoadH<SRC == TR_LIFT> lh;
-    const TrIn in;
-    float wp[8];
+struct TrLoad {
+    TrIn in;
+    float w[8], b[8];
     int t;
-    __device__ __forceinline__ LoadV(const TrIn &i, int t_) : lh(i.h, i.f, i.wl, i.bl, t_), in(i), t(t_) {
-        if (SRC == TR_DOUT)
-            for (int j = 0; j < 8; ++j) wp[j] = i.wp[8 * t_ + j];
-    }
-    __device__ __forceinline__ void operator()(long long p, bool ok, float (&v)[8]) const {
-        if (SRC == TR_H || SRC == TR_LIFT) {
-            const uint4 o = lh(p, ok);
-            const uint32_t w[4] = {o.x, o.y, o.z, o.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                v[2 * j] = bf_lo(w[j]);
-                v[2 * j + 1] = bf_hi(w[j]);
+    __device__ __forceinline__ TrLoad(const TrIn &i, int t_) : in(i), t(t_) {
+        if (SRC == TR_LIFT || SRC == TR_DOUT)
+            for (int j = 0; j < 8; ++j) {
+                w[j] = (SRC == TR_LIFT ? i.wl : i.wp)[8 * t_ + j];
+                b[j] = SRC == TR_LIFT ? i.bl[8 * t_ + j] : 0.0f;
             }
-        } else if (SRC == TR_DOUT) {
-            const float d = ok ? in.dh[p] : 0.0f;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = d * wp[j];
+    }
+    // slot: this lane's first piece of the step; pieces are 32 lanes apart
+    __device__ __forceinline__ void issue(uint4 *slot, long long p, bool ok) const {
+        if (!ok) p = 0;
+        if (SRC == TR_H) {
+            copy16(slot, in.h + p * 32 + 8 * t, ok);
+        } else if (SRC == TR_DZ) {
+            copy16(slot, in.dh + p * 32 + 8 * t, ok);
+            copy16(slot + 32, in.dh + p * 32 + 8 * t + 4, ok);
+            copy16(slot + 64, in.z + p * 32 + 8 * t, ok);
         } else {
+            copy4(slot, (SRC == TR_LIFT ? in.f : in.dh) + p, ok);
+        }
+    }
+    // BF16 pairs of the input (SRC H, LIFT); nodes past the row's end are zero
+    __device__ __forceinline__ uint4 octet(const uint4 *slot, bool ok) const {
+        if (SRC == TR_H) return *slot;
+        const float x = *reinterpret_cast<const float *>(slot);
+        uint4 v;
+        v.x = pack_bf16(fmaf(x, w[0], b[0]), fmaf(x, w[1], b[1]));
+        v.y = pack_bf16(fmaf(x, w[2], b[2]), fmaf(x, w[3], b[3]));
+        v.z = pack_bf16(fmaf(x, w[4], b[4]), fmaf(x, w[5], b[5]));
+        v.w = pack_bf16(fmaf(x, w[6], b[6]), fmaf(x, w[7], b[7]));
+        return ok ? v : make_uint4(0, 0, 0, 0);
+    }
+    __device__ __forceinline__ void values(const uint4 *slot, bool ok, float2 (&v)[4]) const {
+        if (SRC == TR_H || SRC == TR_LIFT) {
+            const uint4 o = octet(slot, ok);
+            v[0] = make_float2(bf_lo(o.x), bf_hi(o.x));
+            v[1] = make_float2(bf_lo(o.y), bf_hi(o.y));
+            v[2] = make_float2(bf_lo(o.z), bf_hi(o.z));
+            v[3] = make_float2(bf_lo(o.w), bf_hi(o.w));
+        } else if (SRC == TR_DOUT) {
+            const float d = *reinterpret_cast<const float *>(slot);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = 0.0f;
-            if (!ok) return;
-            const float4 d0 = *reinterpret_cast<const float4 *>(in.dh + p * 32 + 8 * t);
-            const float4 d1 = *reinterpret_cast<const float4 *>(in.dh + p * 32 + 8 * t + 4);
-            const uint4 o = *reinterpret_cast<const uint4 *>(in.z + p * 32 + 8 * t);
-            v[0] = d0.x * tr_gelu_grad(bf_lo(o.x));
-            v[1] = d0.y * tr_gelu_grad(bf_hi(o.x));
-            v[2] = d0.z * tr_gelu_grad(bf_lo(o.y));
-            v[3] = d0.w * tr_gelu_grad(bf_hi(o.y));
-            v[4] = d1.x * tr_gelu_grad(bf_lo(o.z));
-            v[5] = d1.y * tr_gelu_grad(bf_hi(o.z));
-            v[6] = d1.z * tr_gelu_grad(bf_lo(o.w));
-            v[7] = d1.w * tr_gelu_grad(bf_hi(o.w));
+            for (int j = 0; j < 4; ++j) v[j] = make_float2(d * w[2 * j], d * w[2 * j + 1]);
+        } else {   // zeros past the row's end: dh is zero there
+            const float4 d0 = *reinterpret_cast<const float4 *>(slot), d1 = *reinterpret_cast<const float4 *>(slot + 32);
+            const uint4 o = slot[64];
+            v[0] = make_float2(d0.x * tr_gelu_grad(bf_lo(o.x)), d0.y * tr_gelu_grad(bf_hi(o.x)));
+            v[1] = make_float2(d0.z * tr_gelu_grad(bf_lo(o.y)), d0.w * tr_gelu_grad(bf_hi(o.y)));
+            v[2] = make_float2(d1.x * tr_gelu_grad(bf_lo(o.z)), d1.y * tr_gelu_grad(bf_hi(o.z)));
+            v[3] = make_float2(d1.z * tr_gelu_grad(bf_lo(o.w)), d1.w * tr_gelu_grad(bf_hi(o.w)));
         }
     }
 };
 
-// t2[plane][ky][kx][c] = sum_y sum_x B[y][ky] B[x][kx] v[plane][y][x][c], one CTA per plane
-// (b, z). basis: [G][M]; MP = M rounded up to even (the extra mode is zero).
+// The steps of one warp: rows y0, y0 + dy, .. below y1 of one plane, `per` x steps each.
+struct TrSteps {
+    long long plane;   // first row's index of the plane
+    int y, x, dy, y1, dx, G;
+    __device__ __forceinline__ bool done() const { return y >= y1; }
+    __device__ __forceinline__ long long row() const { return (plane + y) * G; }
+    __device__ __forceinline__ void next() {
+        x += dx;
+        if (x >= G) {
+            x = 0;
+            y += dy;
+        }
+    }
+};
+
+constexpr int kTrDepthA = 8;   // steps of eight nodes in flight per warp (analysis)
+constexpr int kTrParts = 4;    // CTAs per plane
+
+template <int MP, int SRC>
+__host__ __device__ constexpr int tr_analysis_smem() {
+    const int ring = 8 * kTrDepthA * tr_pieces(SRC) * 32 * 16, sums = 8 * MP * MP * 32 * 4;
+    return (ring > sums ? ring : sums) + 256 * MP * 8;
+}
+
+// t2[plane][part][ky][kx][c] = sum_y sum_x B[y][ky] B[x][kx] v[plane][y][x][c] over the part's
+// rows, kTrParts CTAs per plane (b, z). basis: [G][M]; MP = M rounded up to even (the extra mode
+// is zero).
 template <int MP, int SRC>
 __global__ void __launch_bounds__(256, 2) k_tr_analysis(const TrIn in, const float *__restrict__ basis, int G, int M,
                                                         float *__restrict__ t2) {
-    __shared__ float sB[256 * MP];
-    __shared__ float sQ[MP * MP * 32];
+    extern __shared__ __align__(16) uint8_t tr_smem[];
+    float2 *sB = reinterpret_cast<float2 *>(tr_smem);               // (b, b) pairs: packed multiply-adds
+    uint4 *ring = reinterpret_cast<uint4 *>(tr_smem + 256 * MP * 8);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    constexpr int kPieces = tr_pieces(SRC);
+    uint4 *mine = ring + warp * kTrDepthA * kPieces * 32 + lane;
+    const TrLoad<SRC> load(in, t);
+    const int plane = blockIdx.x / kTrParts, part = blockIdx.x % kTrParts;
+    TrSteps ahead{(long long)plane * G, G * part / kTrParts + warp, 0, 8, G * (part + 1) / kTrParts, 8, G};
+    TrSteps at = ahead;
+    int slot = 0;
+    auto issue = [&](int sl) {
+        if (!ahead.done()) load.issue(mine + sl * kPieces * 32, ahead.row() + ahead.x + g, ahead.x + g < G);
+        ahead.next();
+        copy_commit();
+    };
+#pragma unroll
+    for (int i = 0; i < kTrDepthA - 1; ++i) issue(i);
     for (int e = threadIdx.x; e < MP * G; e += 256) {
         const int x = e / MP, k = e % MP;
-        sB[e] = (k < M) ? basis[x * M + k] : 0.0f;
+        const float v = (k < M) ? basis[x * M + k] : 0.0f;
+        sB[e] = make_float2(v, v);
     }
-    for (int e = threadIdx.x; e < MP * MP * 32; e += 256) sQ[e] = 0.0f;
     __syncthreads();
-    const LoadV<SRC> load(in, t);
     float Q[MP][MP];
 #pragma unroll
     for (int a = 0; a < MP; ++a)
 #pragma unroll
         for (int k = 0; k < MP; ++k) Q[a][k] = 0.0f;
-    for (int y = warp; y < G; y += 8) {
-        const long long row = ((long long)blockIdx.x * G + y) * G;
-        float acc[MP][8];
+    while (!at.done()) {
+        const int y = at.y;
+        float2 acc[MP][4];
 #pragma unroll
         for (int k = 0; k < MP; ++k)
 #pragma unroll
-            for (int j = 0; j < 8; ++j) acc[k][j] = 0.0f;
-#pragma unroll 4
+            for (int j = 0; j < 4; ++j) acc[k][j] = make_float2(0.0f, 0.0f);
         for (int x0 = 0; x0 < G; x0 += 8) {
+            copy_wait<kTrDepthA - 2>();
             const int x = x0 + g;
-            float v[8];
-            load(row + x, x < G, v);
-            const float *b = sB + min(x, G - 1) * MP;
+            float2 v[4];
+            load.values(mine + slot * kPieces * 32, x < G, v);
+            issue(slot == 0 ? kTrDepthA - 1 : slot - 1);
+            slot = (slot + 1) & (kTrDepthA - 1);
+            const float2 *b = sB + min(x, G - 1) * MP;
 #pragma unroll
-            for (int k = 0; k < MP; ++k)
+            for (int k = 0; k < MP; ++k) {
+                const float2 bk = b[k];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) acc[k][j] = fmaf(b[k], v[j], acc[k][j]);
+                for (int j = 0; j < 4; ++j) acc[k][j] = __ffma2_rn(bk, v[j], acc[k][j]);
+            }
         }
+        at.x = 0;
+        at.y += 8;
         // sum over the eight g lanes, halving the channels a lane holds each time
         const bool u2 = lane & 16, u1 = lane & 8, u0 = lane & 4;
         float T[MP];
 #pragma unroll
         for (int k = 0; k < MP; ++k) {
+            const float c8[8] = {acc[k][0].x, acc[k][0].y, acc[k][1].x, acc[k][1].y,
+                                 acc[k][2].x, acc[k][2].y, acc[k][3].x, acc[k][3].y};
             float r4[4], r2[2];
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-                r4[j] = (u2 ? acc[k][j + 4] : acc[k][j]) + __shfl_xor_sync(0xffffffffu, u2 ? acc[k][j] : acc[k][j + 4], 16);
+                r4[j] = (u2 ? c8[j + 4] : c8[j]) + __shfl_xor_sync(0xffffffffu, u2 ? c8[j] : c8[j + 4], 16);
 #pragma unroll
             for (int j = 0; j < 2; ++j)
                 r2[j] = (u1 ? r4[j + 2] : r4[j]) + __shfl_xor_sync(0xffffffffu, u1 ? r4[j] : r4[j + 2], 8);
@@ -212,52 +271,79 @@ __global__ void __launch_bounds__(256, 2) k_tr_analysis(const TrIn in, const flo
         }
 #pragma unroll
         for (int a = 0; a < MP; ++a) {
-            const float b = sB[y * MP + a];
+            const float b = sB[y * MP + a].x;
 #pragma unroll
             for (int k = 0; k < MP; ++k) Q[a][k] = fmaf(b, T[k], Q[a][k]);
         }
     }
+    copy_wait<0>();
+    __syncthreads();
+    // the warps' sums in a fixed order; the ring's memory holds them
+    float *sQ = reinterpret_cast<float *>(ring);
     const int c = 8 * t + 4 * ((lane >> 4) & 1) + 2 * ((lane >> 3) & 1) + ((lane >> 2) & 1);   // this lane's channel
-    for (int w = 0; w < 8; ++w) {   // the warps' sums in a fixed order
-        if (warp == w)
 #pragma unroll
-            for (int a = 0; a < MP; ++a)
+    for (int a = 0; a < MP; ++a)
 #pragma unroll
-                for (int k = 0; k < MP; ++k) sQ[(a * MP + k) * 32 + c] += Q[a][k];
-        __syncthreads();
-    }
+        for (int k = 0; k < MP; ++k) sQ[(warp * MP * MP + a * MP + k) * 32 + c] = Q[a][k];
+    __syncthreads();
     float *o = t2 + (long long)blockIdx.x * MP * MP * 32;
-    for (int e = threadIdx.x; e < MP * MP * 32; e += 256) o[e] = sQ[e];
+    for (int e = threadIdx.x; e < MP * MP * 32; e += 256) {
+        float v = 0.0f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) v += sQ[w * MP * MP * 32 + e];
+        o[e] = v;
+    }
 }
 
-// The z analysis of one mode k = (kz, ky, kx), all samples (one warp each): lane = channel.
-__device__ __forceinline__ float z_analysis(const float *__restrict__ t2, const float *__restrict__ basis, int b, int G,
-                                            int M, int MP, int k, int lane) {
+// The z analysis of one mode k = (kz, ky, kx) for eight samples b0 .. b0 + 7: the warps take
+// every eighth plane (all their loads independent: with one warp walking all planes of a sample
+// this waited on memory), lane = channel; warp w returns sample b0 + w.
+__device__ __forceinline__ float z_analysis(const float *__restrict__ t2, const float *__restrict__ basis, int b0, int B,
+                                            int G, int M, int MP, int k, float (*red)[8][32]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int kz = k / (M * M), ky = k / M % M, kx = k % M;
-    const float *p = t2 + ((long long)b * G * MP * MP + ky * MP + kx) * 32 + lane;
     const int stride = MP * MP * 32;
-    float a0 = 0.0f, a1 = 0.0f;
+    __syncthreads();
+#pragma unroll 2
+    for (int i = 0; i < 8; ++i) {
+        if (b0 + i >= B) break;
+        const float *p = t2 + (long long)(b0 + i) * G * kTrParts * stride + (ky * MP + kx) * 32 + lane;
+        float a = 0.0f;
 #pragma unroll 4
-    for (int z = 0; z + 1 < G; z += 2) {
-        a0 = fmaf(__ldg(basis + z * M + kz), __ldg(p + (long long)z * stride), a0);
-        a1 = fmaf(__ldg(basis + (z + 1) * M + kz), __ldg(p + (long long)(z + 1) * stride), a1);
+        for (int z = warp; z < G; z += 8) {
+            const float *q = p + (long long)z * kTrParts * stride;
+            float v = 0.0f;
+#pragma unroll
+            for (int r = 0; r < kTrParts; ++r) v += __ldg(q + r * stride);
+            a = fmaf(__ldg(basis + z * M + kz), v, a);
+        }
+        red[i][warp][lane] = a;
     }
-    if (G & 1) a0 = fmaf(__ldg(basis + (G - 1) * M + kz), __ldg(p + (long long)(G - 1) * stride), a0);
-    return a0 + a1;
+    __syncthreads();
+    float s = 0.0f;
+    if (b0 + warp < B)
+#pragma unroll
+        for (int w = 0; w < 8; ++w) s += red[warp][w][lane];
+    return s;
 }
 
 // hh[b][k][c], g[b][k][o] = sum_i hh[b][k][i] R[k][i][o]; one CTA per mode.
 __global__ void __launch_bounds__(256) k_tr_mix(const float *__restrict__ t2, const float *__restrict__ basis, int B,
                                                 int G, int M, int MP, const float *__restrict__ R,
                                                 float *__restrict__ hh, float *__restrict__ g) {
+    __shared__ float red[8][8][32];
     const int lane = threadIdx.x & 31, k = blockIdx.x, K = gridDim.x;
-    for (int b = threadIdx.x >> 5; b < B; b += 8) {
-        const float v = z_analysis(t2, basis, b, G, M, MP, k, lane);
+    float r[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) r[i] = __ldg(R + (long long)k * 1024 + i * 32 + lane);
+    for (int b0 = 0; b0 < B; b0 += 8) {
+        const float v = z_analysis(t2, basis, b0, B, G, M, MP, k, red);
+        const int b = b0 + (threadIdx.x >> 5);
+        if (b >= B) continue;
         hh[((long long)b * K + k) * 32 + lane] = v;
         float s = 0.0f;
-#pragma unroll 8
-        for (int i = 0; i < 32; ++i)
-            s = fmaf(__shfl_sync(0xffffffffu, v, i), __ldg(R + (long long)k * 1024 + i * 32 + lane), s);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) s = fmaf(__shfl_sync(0xffffffffu, v, i), r[i], s);
         g[((long long)b * K + k) * 32 + lane] = s;
     }
 }
@@ -268,11 +354,14 @@ __global__ void __launch_bounds__(256) k_tr_mix_bwd(const float *__restrict__ t2
                                                     int G, int M, int MP, const float *__restrict__ R,
                                                     const float *__restrict__ hh, float *__restrict__ dhh,
                                                     float *__restrict__ dR) {
-    __shared__ float sR[32 * 33], sdg[64 * 32], shh[64 * 32];
+    __shared__ float sR[32 * 33], sdg[64 * 32], shh[64 * 32], red[8][8][32];
     const int lane = threadIdx.x & 31, k = blockIdx.x, K = gridDim.x;
     for (int e = threadIdx.x; e < 1024; e += 256) sR[(e >> 5) * 33 + (e & 31)] = R[(long long)k * 1024 + e];
-    for (int b = threadIdx.x >> 5; b < B; b += 8) {
-        sdg[b * 32 + lane] = z_analysis(t2, basis, b, G, M, MP, k, lane);
+    for (int b0 = 0; b0 < B; b0 += 8) {
+        const float v = z_analysis(t2, basis, b0, B, G, M, MP, k, red);
+        const int b = b0 + (threadIdx.x >> 5);
+        if (b >= B) continue;
+        sdg[b * 32 + lane] = v;
         shh[b * 32 + lane] = hh[((long long)b * K + k) * 32 + lane];
     }
     __syncthreads();
@@ -353,6 +442,12 @@ struct TrFwd {
     double *loss;
 };
 
+constexpr int kTrDepthF = 5, kTrDepthB = 3;   // steps of 16 nodes in flight per warp
+constexpr int tr_fwd_smem() { return 8 * kTrDepthF * 2 * 32 * 16; }
+constexpr int tr_bwd_smem(bool first, bool last) {
+    return 4 * kTrDepthB * 2 * (tr_pieces(last ? TR_DOUT : TR_DZ) + tr_pieces(first ? TR_LIFT : TR_H)) * 32 * 16;
+}
+
 template <int MP, bool LIFT, bool LAST>
 __global__ void __launch_bounds__(256, 2) k_tr_fwd(const TrFwd a) {
     __shared__ float sB[256 * MP];
@@ -366,7 +461,9 @@ __global__ void __launch_bounds__(256, 2) k_tr_fwd(const TrFwd a) {
         sB[e] = (k < M) ? a.basis[x * M + k] : 0.0f;
     }
     load_fragments(sW, a.W, false, 256);
-    const LoadH<LIFT> load(a.in.h, a.in.f, a.in.wl, a.in.bl, t);
+    extern __shared__ __align__(16) uint8_t tr_smem[];
+    uint4 *mine = reinterpret_cast<uint4 *>(tr_smem) + warp * kTrDepthF * 2 * 32 + lane;
+    const TrLoad<LIFT ? TR_LIFT : TR_H> load(a.in, t);
     float bias[8], wp[LAST ? 8 : 1], gw[LAST ? 8 : 1], gb = 0.0f, bp = 0.0f, inv = 0.0f;
     double loss = 0.0;
 #pragma unroll
@@ -384,26 +481,34 @@ __global__ void __launch_bounds__(256, 2) k_tr_fwd(const TrFwd a) {
     const int items = a.B * G * chunks;
     for (int it = blockIdx.x; it < items; it += gridDim.x) {
         const int plane = it / chunks, y0 = (it % chunks) * kTrRows, y1 = min(y0 + kTrRows, G);
+        TrSteps ahead{(long long)plane * G, y0 + warp, 0, 8, y1, 16, G};
+        int slot = 0;
+        auto issue = [&](int sl) {
+            if (!ahead.done()) {
+                load.issue(mine + sl * 64, ahead.row() + ahead.x + g, ahead.x + g < G);
+                load.issue(mine + sl * 64 + 32, ahead.row() + ahead.x + 8 + g, ahead.x + 8 + g < G);
+            }
+            ahead.next();
+            copy_commit();
+        };
+        for (int i = 0; i < kTrDepthF - 1; ++i) issue(i);
         __syncthreads();
         z_synthesis<MP>(sS, sB, a.g, plane / G, plane % G, M, 256);
         __syncthreads();
         for (int y = y0 + warp; y < y1; y += 8) {
             y_synthesis<MP>(sT[warp], sS, sB, y, lane);
-            float T[MP][8];
+            float2 T[MP][4];
 #pragma unroll
-            for (int k = 0; k < MP; ++k) {
-                const float4 u = *reinterpret_cast<const float4 *>(sT[warp] + k * 32 + 8 * t);
-                const float4 v = *reinterpret_cast<const float4 *>(sT[warp] + k * 32 + 8 * t + 4);
-                T[k][0] = u.x, T[k][1] = u.y, T[k][2] = u.z, T[k][3] = u.w;
-                T[k][4] = v.x, T[k][5] = v.y, T[k][6] = v.z, T[k][7] = v.w;
-            }
+            for (int k = 0; k < MP; ++k)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) T[k][j] = *reinterpret_cast<const float2 *>(sT[warp] + k * 32 + 8 * t + 2 * j);
             const long long row = ((long long)plane * G + y) * G;
-            uint4 hA = load(row + g, g < G), hB = load(row + 8 + g, 8 + g < G);
             for (int x0 = 0; x0 < G; x0 += 16) {
-                const uint4 cA = hA, cB = hB;
-                const int xn = x0 + 16 + g;
-                hA = load(row + xn, xn < G);
-                hB = load(row + xn + 8, xn + 8 < G);
+                copy_wait<kTrDepthF - 2>();
+                const uint4 cA = load.octet(mine + slot * 64, x0 + g < G);
+                const uint4 cB = load.octet(mine + slot * 64 + 32, x0 + 8 + g < G);
+                issue(slot == 0 ? kTrDepthF - 1 : slot - 1);
+                slot = slot == kTrDepthF - 1 ? 0 : slot + 1;
                 float d[4][4];
 #pragma unroll
                 for (int n = 0; n < 4; ++n) d[n][0] = d[n][1] = d[n][2] = d[n][3] = 0.0f;
@@ -423,16 +528,17 @@ __global__ void __launch_bounds__(256, 2) k_tr_fwd(const TrFwd a) {
                 for (int r = 0; r < 2; ++r) {
                     const int x = x0 + 8 * r + g;
                     const bool ok = x < G;
-                    float s[8];
+                    float2 s2[4];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) s[j] = bias[j];
+                    for (int j = 0; j < 4; ++j) s2[j] = make_float2(bias[2 * j], bias[2 * j + 1]);
                     const float *b = sB + min(x, G - 1) * MP;
 #pragma unroll
                     for (int k = 0; k < MP; ++k)
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) s[j] = fmaf(b[k], T[k][j], s[j]);
+                        for (int j = 0; j < 4; ++j) s2[j] = __ffma2_rn(make_float2(b[k], b[k]), T[k][j], s2[j]);
+                    float s[8];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) s[j] += d[j >> 1][2 * r + (j & 1)];
+                    for (int j = 0; j < 8; ++j) s[j] = (j & 1 ? s2[j >> 1].y : s2[j >> 1].x) + d[j >> 1][2 * r + (j & 1)];
                     const long long p = row + x;
                     uint4 o;
                     if (LAST || a.z != nullptr) {
@@ -475,6 +581,7 @@ __global__ void __launch_bounds__(256, 2) k_tr_fwd(const TrFwd a) {
         }
     }
     if constexpr (LAST) {
+        copy_wait<0>();
         if (a.target == nullptr) return;
         // the projection's gradients and the loss: lanes of one t, then the warps
 #pragma unroll
@@ -522,8 +629,12 @@ __global__ void __launch_bounds__(128, 3) k_tr_bwd(const TrBwd a) {
         sB[e] = (k < M) ? a.basis[x * M + k] : 0.0f;
     }
     load_fragments(sW, a.W, true, 128);
-    const LoadH<FIRST> load_h(a.in.h, a.in.f, a.in.wl, a.in.bl, t);
-    const LoadV<LAST ? TR_DOUT : TR_DZ> load_dz(a.in, t);
+    constexpr int kH = FIRST ? TR_LIFT : TR_H, kZ = LAST ? TR_DOUT : TR_DZ;
+    constexpr int kStep = 2 * (tr_pieces(kZ) + tr_pieces(kH)) * 32;   // ring slots of a step
+    extern __shared__ __align__(16) uint8_t tr_smem[];
+    uint4 *mine = reinterpret_cast<uint4 *>(tr_smem) + warp * kTrDepthB * kStep + lane;
+    const TrLoad<kH> load_h(a.in, t);
+    const TrLoad<kZ> load_dz(a.in, t);
     float dW[2][4][4], db[8], gl[FIRST ? 8 : 1], gbl[FIRST ? 8 : 1];
 #pragma unroll
     for (int m = 0; m < 2; ++m)
@@ -538,6 +649,22 @@ __global__ void __launch_bounds__(128, 3) k_tr_bwd(const TrBwd a) {
     const int items = a.B * G * chunks;
     for (int it = blockIdx.x; it < items; it += gridDim.x) {
         const int plane = it / chunks, y0 = (it % chunks) * kTrRows, y1 = min(y0 + kTrRows, G);
+        TrSteps ahead{(long long)plane * G, y0 + warp, 0, 4, y1, 16, G};
+        int slot = 0;
+        auto issue = [&](int sl) {
+            if (!ahead.done()) {
+                uint4 *q = mine + sl * kStep;
+                const long long p = ahead.row() + ahead.x + g;
+                const bool okA = ahead.x + g < G, okB = ahead.x + 8 + g < G;
+                load_dz.issue(q, p, okA);
+                load_dz.issue(q + tr_pieces(kZ) * 32, p + 8, okB);
+                load_h.issue(q + 2 * tr_pieces(kZ) * 32, p, okA);
+                load_h.issue(q + 2 * tr_pieces(kZ) * 32 + 32, p + 8, okB);
+            }
+            ahead.next();
+            copy_commit();
+        };
+        for (int i = 0; i < kTrDepthB - 1; ++i) issue(i);
         __syncthreads();
         z_synthesis<MP>(sS, sB, a.dhh, plane / G, plane % G, M, 128);
         __syncthreads();
@@ -546,20 +673,26 @@ __global__ void __launch_bounds__(128, 3) k_tr_bwd(const TrBwd a) {
             const long long row = ((long long)plane * G + y) * G;
             for (int x0 = 0; x0 < G; x0 += 16) {
                 const int xA = x0 + g, xB = x0 + 8 + g;
-                float vA[8], vB[8];
-                load_dz(row + xA, xA < G, vA);
-                load_dz(row + xB, xB < G, vB);
-                const uint4 oA = load_h(row + xA, xA < G), oB = load_h(row + xB, xB < G);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) db[j] += vA[j] + vB[j];
+                copy_wait<kTrDepthB - 2>();
+                const uint4 *q = mine + slot * kStep;
+                float2 vA[4], vB[4];
+                load_dz.values(q, xA < G, vA);
+                load_dz.values(q + tr_pieces(kZ) * 32, xB < G, vB);
+                const uint4 oA = load_h.octet(q + 2 * tr_pieces(kZ) * 32, xA < G);
+                const uint4 oB = load_h.octet(q + 2 * tr_pieces(kZ) * 32 + 32, xB < G);
+                issue(slot == 0 ? kTrDepthB - 1 : slot - 1);
+                slot = slot == kTrDepthB - 1 ? 0 : slot + 1;
                 uint32_t lA[3][4], lB[3][4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
+                for (int j = 0; j < 4; ++j) {
+                    db[2 * j] += vA[j].x + vB[j].x;
+                    db[2 * j + 1] += vA[j].y + vB[j].y;
 #pragma unroll
                     for (int l = 0; l < 3; ++l) {
-                        lA[l][j] = take_level(vA[2 * j], vA[2 * j + 1]);
-                        lB[l][j] = take_level(vB[2 * j], vB[2 * j + 1]);
+                        lA[l][j] = take_level(vA[j].x, vA[j].y);
+                        lB[l][j] = take_level(vB[j].x, vB[j].y);
                     }
+                }
                 // dW += h^T dz over the 16 nodes
                 {
                     const uint32_t hA[4] = {oA.x, oA.y, oA.z, oA.w}, hB[4] = {oB.x, oB.y, oB.z, oB.w};
@@ -605,38 +738,40 @@ __global__ void __launch_bounds__(128, 3) k_tr_bwd(const TrBwd a) {
                                          lB[l][2 * ks + 1], w.z, w.w);
                             }
                         }
-                float s[2][8];
+                float2 s2[2][4];
                 const float *bA = sB + min(xA, G - 1) * MP, *bB = sB + min(xB, G - 1) * MP;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) s[0][j] = s[1][j] = 0.0f;
+                for (int j = 0; j < 4; ++j) s2[0][j] = s2[1][j] = make_float2(0.0f, 0.0f);
 #pragma unroll
                 for (int k = 0; k < MP; ++k) {
                     const float4 u = *reinterpret_cast<const float4 *>(sT[warp] + k * 32 + 8 * t);
                     const float4 v = *reinterpret_cast<const float4 *>(sT[warp] + k * 32 + 8 * t + 4);
-                    const float T[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+                    const float2 T[4] = {{u.x, u.y}, {u.z, u.w}, {v.x, v.y}, {v.z, v.w}};
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        s[0][j] = fmaf(bA[k], T[j], s[0][j]);
-                        s[1][j] = fmaf(bB[k], T[j], s[1][j]);
+                    for (int j = 0; j < 4; ++j) {
+                        s2[0][j] = __ffma2_rn(make_float2(bA[k], bA[k]), T[j], s2[0][j]);
+                        s2[1][j] = __ffma2_rn(make_float2(bB[k], bB[k]), T[j], s2[1][j]);
                     }
                 }
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
                     const int x = x0 + 8 * r + g;
+                    float s[8];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) s[r][j] += d[j >> 1][2 * r + (j & 1)];
+                    for (int j = 0; j < 8; ++j)
+                        s[j] = (j & 1 ? s2[r][j >> 1].y : s2[r][j >> 1].x) + d[j >> 1][2 * r + (j & 1)];
                     if (x >= G) continue;
                     if constexpr (FIRST) {
                         const float fv = a.in.f[row + x];
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
-                            gl[j] = fmaf(fv, s[r][j], gl[j]);
-                            gbl[j] += s[r][j];
+                            gl[j] = fmaf(fv, s[j], gl[j]);
+                            gbl[j] += s[j];
                         }
                     } else {
                         float4 *o = reinterpret_cast<float4 *>(a.dh_prev + (row + x) * 32 + 8 * t);
-                        o[0] = make_float4(s[r][0], s[r][1], s[r][2], s[r][3]);
-                        o[1] = make_float4(s[r][4], s[r][5], s[r][6], s[r][7]);
+                        o[0] = make_float4(s[0], s[1], s[2], s[3]);
+                        o[1] = make_float4(s[4], s[5], s[6], s[7]);
                     }
                 }
             }
@@ -698,6 +833,30 @@ struct TrNet {
     long long off_wp;
 };
 
+template <typename K>
+int tr_opt_in(K kernel, int bytes) {
+    QN_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    return QN_OK;
+}
+
+// More than 48 KB of shared memory for every kernel of one MP (at network creation).
+template <int MP>
+int tr_set_attributes() {
+    int rc = tr_opt_in(k_tr_analysis<MP, TR_H>, tr_analysis_smem<MP, TR_H>());
+    if (rc == QN_OK) rc = tr_opt_in(k_tr_analysis<MP, TR_LIFT>, tr_analysis_smem<MP, TR_LIFT>());
+    if (rc == QN_OK) rc = tr_opt_in(k_tr_analysis<MP, TR_DZ>, tr_analysis_smem<MP, TR_DZ>());
+    if (rc == QN_OK) rc = tr_opt_in(k_tr_analysis<MP, TR_DOUT>, tr_analysis_smem<MP, TR_DOUT>());
+    if (rc == QN_OK) rc = tr_opt_in(k_tr_fwd<MP, false, false>, tr_fwd_smem());
+    if (rc == QN_OK) rc = tr_opt_in(k_tr_fwd<MP, false, true>, tr_fwd_smem());
+    if (rc == QN_OK) rc = tr_opt_in(k_tr_fwd<MP, true, false>, tr_fwd_smem());
+    if (rc == QN_OK) rc = tr_opt_in(k_tr_fwd<MP, true, true>, tr_fwd_smem());
+    if (rc == QN_OK) rc = tr_opt_in(k_tr_bwd<MP, false, false>, tr_bwd_smem(false, false));
+    if (rc == QN_OK) rc = tr_opt_in(k_tr_bwd<MP, false, true>, tr_bwd_smem(false, true));
+    if (rc == QN_OK) rc = tr_opt_in(k_tr_bwd<MP, true, false>, tr_bwd_smem(true, false));
+    if (rc == QN_OK) rc = tr_opt_in(k_tr_bwd<MP, true, true>, tr_bwd_smem(true, true));
+    return rc;
+}
+
 template <int MP>
 void tr_forward(const TrNet &n, cudaStream_t s) {
     const int planes = n.B * n.G, K = n.M * n.M * n.M;
@@ -710,9 +869,9 @@ void tr_forward(const TrNet &n, cudaStream_t s) {
         a.in.wl = n.params;
         a.in.bl = n.params + 32;
         if (l == 0)
-            k_tr_analysis<MP, TR_LIFT><<<planes, 256, 0, s>>>(a.in, n.basis, n.G, n.M, n.t2);
+            k_tr_analysis<MP, TR_LIFT><<<planes * kTrParts, 256, tr_analysis_smem<MP, TR_LIFT>(), s>>>(a.in, n.basis, n.G, n.M, n.t2);
         else
-            k_tr_analysis<MP, TR_H><<<planes, 256, 0, s>>>(a.in, n.basis, n.G, n.M, n.t2);
+            k_tr_analysis<MP, TR_H><<<planes * kTrParts, 256, tr_analysis_smem<MP, TR_H>(), s>>>(a.in, n.basis, n.G, n.M, n.t2);
         k_tr_mix<<<K, 256, 0, s>>>(n.t2, n.basis, n.B, n.G, n.M, MP, n.params + n.off_R[l], n.hh[l], n.g);
         a.basis = n.basis;
         a.g = n.g;
@@ -733,13 +892,13 @@ void tr_forward(const TrNet &n, cudaStream_t s) {
         a.loss = n.loss;
         const bool last = l == n.L - 1;
         if (l == 0 && last)
-            k_tr_fwd<MP, true, true><<<grid, 256, 0, s>>>(a);
+            k_tr_fwd<MP, true, true><<<grid, 256, tr_fwd_smem(), s>>>(a);
         else if (l == 0)
-            k_tr_fwd<MP, true, false><<<grid, 256, 0, s>>>(a);
+            k_tr_fwd<MP, true, false><<<grid, 256, tr_fwd_smem(), s>>>(a);
         else if (last)
-            k_tr_fwd<MP, false, true><<<grid, 256, 0, s>>>(a);
+            k_tr_fwd<MP, false, true><<<grid, 256, tr_fwd_smem(), s>>>(a);
         else
-            k_tr_fwd<MP, false, false><<<grid, 256, 0, s>>>(a);
+            k_tr_fwd<MP, false, false><<<grid, 256, tr_fwd_smem(), s>>>(a);
     }
 }
 
@@ -759,9 +918,9 @@ void tr_backward(const TrNet &n, cudaStream_t s) {
         a.in.dh = last ? n.dout : n.dh;
         a.in.wp = n.params + n.off_wp;
         if (last)
-            k_tr_analysis<MP, TR_DOUT><<<planes, 256, 0, s>>>(a.in, n.basis, n.G, n.M, n.t2);
+            k_tr_analysis<MP, TR_DOUT><<<planes * kTrParts, 256, tr_analysis_smem<MP, TR_DOUT>(), s>>>(a.in, n.basis, n.G, n.M, n.t2);
         else
-            k_tr_analysis<MP, TR_DZ><<<planes, 256, 0, s>>>(a.in, n.basis, n.G, n.M, n.t2);
+            k_tr_analysis<MP, TR_DZ><<<planes * kTrParts, 256, tr_analysis_smem<MP, TR_DZ>(), s>>>(a.in, n.basis, n.G, n.M, n.t2);
         k_tr_mix_bwd<<<K, 256, 0, s>>>(n.t2, n.basis, n.B, n.G, n.M, MP, n.params + n.off_R[l], n.hh[l], n.dhh,
                                        n.grads + n.off_R[l]);
         a.basis = n.basis;
@@ -776,13 +935,13 @@ void tr_backward(const TrNet &n, cudaStream_t s) {
         a.G = n.G;
         a.M = n.M;
         if (l == 0 && last)
-            k_tr_bwd<MP, true, true><<<grid, 128, 0, s>>>(a);
+            k_tr_bwd<MP, true, true><<<grid, 128, tr_bwd_smem(true, true), s>>>(a);
         else if (l == 0)
-            k_tr_bwd<MP, true, false><<<grid, 128, 0, s>>>(a);
+            k_tr_bwd<MP, true, false><<<grid, 128, tr_bwd_smem(true, false), s>>>(a);
         else if (last)
-            k_tr_bwd<MP, false, true><<<grid, 128, 0, s>>>(a);
+            k_tr_bwd<MP, false, true><<<grid, 128, tr_bwd_smem(false, true), s>>>(a);
         else
-            k_tr_bwd<MP, false, false><<<grid, 128, 0, s>>>(a);
+            k_tr_bwd<MP, false, false><<<grid, 128, tr_bwd_smem(false, false), s>>>(a);
     }
 }
 
