@@ -160,6 +160,8 @@ struct qn_ctx {
     int *hc0, *hlen;
     double *hval;
     int hbw;
+    int2 *sem_x, *sem_h;   // split solves: fixed-point U and coefficients (k_residual_sem_fixed)
+    int sem_q;
 };
 
 struct StateMirror {
@@ -339,6 +341,8 @@ static void ctx_free(qn_ctx *c) {
     cudaFree(c->hc0);
     cudaFree(c->hlen);
     cudaFree(c->hval);
+    cudaFree(c->sem_x);
+    cudaFree(c->sem_h);
     for (int b = 0; b < 2; ++b) {
         cudaFree(c->w64[b]);
         cudaFree(c->bhi[b]);
@@ -536,6 +540,26 @@ extern "C" int qn_ctx_create(const qn_problem *p, qn_ctx **out) {
         CK(cudaMemcpy(c->hc0, c0.data(), sizeof(int) * n, cudaMemcpyHostToDevice));
         CK(cudaMemcpy(c->hlen, len.data(), sizeof(int) * n, cudaMemcpyHostToDevice));
         CK(cudaMemcpy(c->hval, hv.data(), sizeof(double) * (size_t)n * bw, cudaMemcpyHostToDevice));
+        if (p->precision != QN_PREC_FP64) {
+            // integers H 2^q, q such that every row sums to at most 2^58 in magnitude
+            double most = 0.0;
+            for (int i = 0; i < n; ++i) {
+                double sum = 0.0;
+                for (int j = 0; j < bw; ++j) sum += fabs(hv[(size_t)i * bw + j]);
+                most = fmax(most, sum);
+            }
+            c->sem_q = 57 - ilogb(most);
+            std::vector<int2> hx((size_t)bw * n);
+            for (int i = 0; i < n; ++i)
+                for (int j = 0; j < bw; ++j) {
+                    const long long v = llrint(ldexp(hv[(size_t)i * bw + j], c->sem_q));
+                    const int hi = (int)((v + (1ll << 28)) >> 29);   // high part and balanced low 29 bits
+                    hx[(size_t)j * n + i] = make_int2(hi, (int)(v - ((long long)hi << 29)));
+                }
+            CK(cudaMalloc(&c->sem_h, sizeof(int2) * hx.size()));
+            CK(cudaMemcpy(c->sem_h, hx.data(), sizeof(int2) * hx.size(), cudaMemcpyHostToDevice));
+            CK(cudaMalloc(&c->sem_x, sizeof(int2) * (size_t)c->N));
+        }
     } else if (p->bc == QN_BC_ROBIN) {
         rc = qn_setup_1d_robin(n, c->h, p->robin_kappa, S.data(), Si.data(), lam.data());
         if (rc != QN_OK) {
@@ -880,6 +904,13 @@ static int enqueue_residual(qn_ctx *c, const double *U, const double *f, double 
         rc = launch_residual_mirror(a, c->nparts, c->res_zc, &c->res_parts, s);
     } else if (tiled) {
         rc = launch_residual_tiled(a, c->nparts, c->res_zc, &c->res_parts, s);
+    } else if (split_solve && c->sem_x != nullptr && c->cur_iter >= 1) {
+        a.sem_x = c->sem_x;
+        a.sem_h = c->sem_h;
+        a.sem_q = c->sem_q;
+        a.fx_headroom = &c->st->fx_headroom;
+        rc = launch_residual_sem_fixed(a, c->nparts, &c->res_parts, c->st, c->num_sms, s);
+        c->launches += 4;
     } else {
         rc = launch_residual(a, c->nparts, s);
         c->res_parts = c->nparts;

@@ -78,6 +78,12 @@ struct ResidualArgs {
     const int *hlen;
     const double *hval;
     int hbw;
+    // the integer form of the banded sums (k_residual_sem_fixed): fixed-point values of U,
+    // coefficients [tap][row] scaled by 2^sem_q, DevState::fx_headroom; sem_x == nullptr: FP64
+    int2 *sem_x;
+    const int2 *sem_h;
+    int sem_q;
+    const int *fx_headroom;
     double robin;              // QN_BC_ROBIN: 2 kappa / h, added times u once per face a node lies on
     const DevState *zero_start;  // iteration 0 of a split solve (KIND 0-2): when the preparation pass
                                  // found U_0 = 0 it already wrote the residual -f, so the tiled kernels
@@ -122,6 +128,11 @@ struct GemmShape {
 int launch_residual(const ResidualArgs &a, int grid, cudaStream_t s);
 // spectral elements (qn_sem.cu): the per-node residual with the banded H
 int launch_residual_sem(const ResidualArgs &a, int grid, cudaStream_t s);
+// The same through integer sums (iterations >= 1 of a split solve, ||f|| known): scans max|U|,
+// converts U, and falls back to the FP64 kernel on the device when max|U| is out of range.
+// Five launches.
+int launch_residual_sem_fixed(const ResidualArgs &a, int max_grid, int *grid_used, DevState *st, int num_sms,
+                              cudaStream_t s);
 // 3-D split solve, iterations >= 2: no FP64 arithmetic per point (k_residual_tiled).
 // Uses at most max_grid blocks; the number of partial records written goes to *grid_used.
 int launch_residual_tiled(const ResidualArgs &a, int max_grid, int zchunk, int *grid_used, cudaStream_t s);

@@ -12,8 +12,9 @@
 // Device side (k_residual_sem): the residual A_h U + lam U + b U^3 + V U - f with
 // A_h = sum over axes of H applied along that axis. H is banded (a node couples to
 // the nodes of its one or two elements): row i holds hlen[i] <= 2k+1 values from
-// column hc0[i]. One thread per node, FP64 (the stencil coefficients are not
-// integers, so the exact fixed-point form of the difference stencil does not apply).
+// column hc0[i]. One thread per node. k_residual_sem sums in FP64; the split solve's iterations
+// after the first take k_residual_sem_fixed, which forms the banded sums exactly from 57-bit
+// fixed-point values and coefficients on the integer pipe.
 #include <math.h>
 #include <string.h>
 
@@ -21,6 +22,7 @@
 #include <vector>
 
 #include "qn_internal.h"
+#include "qn_df.cuh"
 #include "qn_numeric.cuh"
 
 namespace qn {
@@ -111,6 +113,7 @@ __device__ Red4s block_red(Red4s v) {
 template <int DIM, bool SPLIT, bool POT>
 __global__ void __launch_bounds__(256) k_residual_sem(ResidualArgs a) {
     if (a.done != nullptr && *(volatile const int *)a.done) return;
+    if (a.sem_x != nullptr && *(volatile const int *)a.fx_e != 0) return;   // k_residual_sem_fixed did it
     const int n = a.n;
     const int P = SPLIT ? a.P : n;
     const long long rows = (DIM == 3) ? (long long)P * P : (long long)P;
@@ -206,6 +209,197 @@ __global__ void __launch_bounds__(256) k_residual_sem(ResidualArgs a) {
         p[2] = acc.mn;
         p[3] = acc.mx;
     }
+}
+
+// ---- the banded sums on the integer pipe ------------------------------------------------
+// The FP64 kernel above is bound by the FP64 pipe (2 lanes per clock per SM): about 21 multiply-
+// adds along the axes and 11 other operations a node at Q^4, 1.03 ms at 255^3. Here every value
+// is an integer X = U 2^(1080 - E) with |X| < 2^56 (E two above the exponent of max|U|, taken by a
+// scan of U first) and every coefficient an integer C = H 2^q whose rows sum to at most 2^58 in
+// magnitude. Both are held as h 2^29 + l with |l| <= 2^28, and a tap is three 32 x 32 + 64-bit
+// multiply-adds: h h' and h l' + l h'. The l l' that are left out have zero mean and are below
+// 2^-57 of the largest value times the row sum together, where a chain of FP64 multiply-adds
+// rounds every partial sum at 2^-53; the two sums join in one 64-bit value that is rounded to
+// FP64 once. The limits hold for all degrees (3 x 33 taps at Q^16).
+constexpr int kSemLo = 29;
+
+__device__ __forceinline__ int2 sem_pair(long long v) {
+    const int h = (int)((v + (1ll << (kSemLo - 1))) >> kSemLo);
+    return make_int2(h, (int)(v - ((long long)h << kSemLo)));
+}
+
+__global__ void __launch_bounds__(256) k_sem_to_fixed(const double *__restrict__ U, long long N, int2 *__restrict__ X,
+                                                      const DevState *__restrict__ st) {
+    if (*(volatile const int *)&st->done || st->fx_e == 0) return;
+    const int E = st->fx_e - st->fx_headroom + 2;
+    unsigned bad = 0;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
+        X[i] = sem_pair(fx_of((unsigned long long)__double_as_longlong(__ldg(U + i)), E, bad));
+}
+
+struct SemSum {
+    long long hh, mid;
+    __device__ __forceinline__ void add(int2 x, int2 c) {
+        hh += (long long)x.x * c.x;
+        mid += (long long)x.x * c.y;
+        mid += (long long)x.y * c.x;
+    }
+};
+
+// A block takes groups of four rows (y .. y + 3 of one z), one thread per x: the x and z
+// coefficients are loaded once for the four, and their sums are independent chains. The y and z
+// coefficients of the group sit in shared memory. KIND 0: general; 1: with a potential; 2:
+// lam = 0 and b = 1 (two FP64 operations a node fewer).
+//
+// Measured at 255^3, Q^4: 0.46 ms with four rows and four blocks per SM (64 registers, 80 bytes
+// spilled), 0.51 with three blocks, 0.48 with two rows; plus 0.07 ms for the scan and the
+// conversion, against 1.03 ms in FP64. It waits on L1 / L2 loads of the neighbours' values.
+constexpr int kSemRows = 4, kSemBlocks = 4;   // blocks per SM
+
+template <int DIM, int KIND>
+__global__ void __launch_bounds__(256, kSemBlocks) k_residual_sem_fixed(const ResidualArgs a) {
+    if (a.done != nullptr && *(volatile const int *)a.done) return;
+    if (*(volatile const int *)a.fx_e == 0) return;   // max|U| out of range: k_residual_sem follows
+    constexpr int kMaxBand = 2 * 16 + 1;
+    __shared__ int2 sc[2][kSemRows + 1][kMaxBand];   // y coefficients of the rows, z coefficients
+    const int n = a.n, P = a.P, bw = a.hbw;
+    const int groups = (P / kSemRows) * ((DIM == 3) ? P : 1);   // P is a multiple of 64
+    const int nn = n * n;                                        // n <= 1024
+    const int E = *a.fx_e - *a.fx_headroom + 2;
+    const int2 *__restrict__ X = a.sem_x;
+    const int2 *__restrict__ H = a.sem_h;   // [tap][row]
+    Red4s acc{0.0, 0.0, INFINITY, -INFINITY};
+    unsigned long long amin = 0x7FFFFFFFFFFFFFFFull, amax = 0ull;
+    const int per = (groups + gridDim.x - 1) / gridDim.x;   // consecutive groups: y neighbours in L1
+    const int g1 = min(groups, (int)(blockIdx.x + 1) * per);
+    // the next group's coefficients are loaded during this one (one thread each: 5 x 33 < 256)
+    const int er = threadIdx.x / bw, ej = threadIdx.x - er * bw;
+    auto coefficient = [&](int grp) -> int2 {
+        const int y = (grp % (P / kSemRows)) * kSemRows, z = grp / (P / kSemRows);
+        if (er > kSemRows || grp >= g1 || y >= n || z >= n) return make_int2(0, 0);
+        return __ldg(H + ej * n + (er < kSemRows ? min(y + er, n - 1) : z));
+    };
+    int2 next = coefficient(blockIdx.x * per);
+    int buf = 0;
+    for (int grp = blockIdx.x * per; grp < g1; ++grp, buf ^= 1) {
+        const int y0 = (grp % (P / kSemRows)) * kSemRows, z = grp / (P / kSemRows);
+        const bool any = y0 < n && (DIM == 2 || z < n);
+        if (er <= kSemRows) sc[buf][er][ej] = next;
+        next = coefficient(grp + 1);
+        __syncthreads();
+        const int2(*sy)[kMaxBand] = sc[buf], *sz = sc[buf][kSemRows];
+        for (int x = threadIdx.x; x < P; x += 256) {
+            double rr[kSemRows] = {};
+            if (any && x < n) {
+                const int c0 = (DIM == 3 ? z * nn : 0) + y0 * n + x;
+                double u[kSemRows], fv[kSemRows];
+                SemSum s[kSemRows] = {};
+                int off[kSemRows];   // the group's rows (rows past the grid repeat the last one)
+#pragma unroll
+                for (int r = 0; r < kSemRows; ++r) {
+                    off[r] = min(r, n - 1 - y0) * n;
+                    u[r] = __ldg(a.U + c0 + off[r]);
+                    fv[r] = __ldg(a.f + c0 + off[r]);
+                }
+                {   // along x: the whole band in every lane (zero coefficients past a row's own,
+                    // columns past the grid read the last one)
+                    const int j0 = __ldg(a.hc0 + x), last = n - 1 - j0;
+                    const int2 *px = X + (c0 - x + j0);
+                    const int2 *hx = H + x;
+#pragma unroll 3
+                    for (int j = 0; j < bw; ++j) {
+                        const int2 c = __ldg(hx + j * n);
+                        const int2 *q = px + min(j, last);
+#pragma unroll
+                        for (int r = 0; r < kSemRows; ++r) s[r].add(__ldg(q + off[r]), c);
+                    }
+                }
+                if (DIM == 3) {   // along z
+                    const int len = __ldg(a.hlen + z);
+                    const int2 *pz = X + (c0 + (__ldg(a.hc0 + z) - z) * nn);
+#pragma unroll 5
+                    for (int j = 0; j < len; ++j) {
+                        const int2 c = sz[j];
+#pragma unroll
+                        for (int r = 0; r < kSemRows; ++r) s[r].add(__ldg(pz + off[r]), c);
+                        pz += nn;
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < kSemRows; ++r) {   // along y
+                    const int y = min(y0 + r, n - 1);
+                    const int len = __ldg(a.hlen + y);
+                    const int2 *py = X + (c0 + (__ldg(a.hc0 + y) - y0) * n);
+#pragma unroll 5
+                    for (int j = 0; j < len; ++j) {
+                        s[r].add(__ldg(py), sy[r][j]);
+                        py += n;
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < kSemRows; ++r) {
+                    if (y0 + r >= n) break;
+                    // sum / 2^54, in units of 2^(E - 1026 - q)
+                    const double lap = fixed_to_double((s[r].hh << 4) + ((s[r].mid + (1ll << 24)) >> 25), E + 54 - a.sem_q);
+                    const double u2 = u[r] * u[r];
+                    double v;
+                    if (KIND == 2) {
+                        v = lap + fma(u2, u[r], -fv[r]);
+                    } else {
+                        double cv = a.lam;
+                        if (KIND == 1) {
+                            cv += __ldg(a.pot + x) + __ldg(a.pot + n + y0 + r);
+                            if (DIM == 3) cv += __ldg(a.pot + 2 * n + z);
+                        }
+                        v = lap + fma(a.b * u2, u[r], fma(cv, u[r], -fv[r]));
+                        if (KIND == 1) {
+                            const double d = fma(3.0 * a.b, u2, cv - a.lam);
+                            acc.mn = fmin(acc.mn, d);
+                            acc.mx = fmax(acc.mx, d);
+                        }
+                    }
+                    acc.r2 = fma(v, v, acc.r2);
+                    if (KIND != 1) {
+                        const unsigned long long ab = abs_bits(u[r]);
+                        amin = ab < amin ? ab : amin;
+                        amax = ab > amax ? ab : amax;
+                    }
+                    rr[r] = v;
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < kSemRows; ++r) {
+                const float rf = d2f_rn(rr[r]);
+                const __nv_bfloat16 hi = __float2bfloat16_rn(rf);
+                const long long o = ((long long)z * P + y0 + r) * P + x;
+                a.Rhi[o] = hi;
+                a.Rlo[o] = __float2bfloat16_rn(rf - __bfloat162float(hi));
+            }
+        }
+    }
+    if (KIND != 1 && amin != 0x7FFFFFFFFFFFFFFFull) {
+        const double lo = __longlong_as_double((long long)amin), hi = __longlong_as_double((long long)amax);
+        acc.mn = lo * lo;
+        acc.mx = hi * hi;
+    }
+    acc = block_red(acc);
+    if (threadIdx.x == 0) {
+        double *p = a.partials + 4ll * blockIdx.x;
+        p[0] = acc.r2;
+        p[1] = 0.0;
+        p[2] = acc.mn;
+        p[3] = acc.mx;
+    }
+}
+
+template <int DIM>
+void launch_sem_fixed_dim(const ResidualArgs &a, int grid, cudaStream_t s) {
+    if (a.pot != nullptr)
+        k_residual_sem_fixed<DIM, 1><<<grid, 256, 0, s>>>(a);
+    else if (a.lam == 0.0 && a.b == 1.0)
+        k_residual_sem_fixed<DIM, 2><<<grid, 256, 0, s>>>(a);
+    else
+        k_residual_sem_fixed<DIM, 0><<<grid, 256, 0, s>>>(a);
 }
 
 template <int DIM, bool SPLIT>
@@ -331,6 +525,22 @@ bool symmetric_eigen(int n, std::vector<double> &A, std::vector<double> &d) {
     }
     d = d2;
     return true;
+}
+
+int launch_residual_sem_fixed(const ResidualArgs &a, int max_grid, int *grid_used, DevState *st, int num_sms,
+                              cudaStream_t s) {
+    const int grid = kSemBlocks * num_sms < max_grid ? kSemBlocks * num_sms : max_grid;
+    *grid_used = grid;
+    const long long N = (long long)a.n * a.n * (a.dim == 3 ? a.n : 1);
+    int rc = launch_umax(a.U, N, st, 2 * num_sms, s);
+    if (rc != QN_OK) return rc;
+    k_sem_to_fixed<<<8 * num_sms, 256, 0, s>>>(a.U, N, a.sem_x, st);
+    if (a.dim == 3)
+        launch_sem_fixed_dim<3>(a, grid, s);
+    else
+        launch_sem_fixed_dim<2>(a, grid, s);
+    QN_CUDA(cudaGetLastError());
+    return launch_residual_sem(a, grid, s);   // returns at once unless max|U| is out of range
 }
 
 int launch_residual_sem(const ResidualArgs &a, int grid, cudaStream_t s) {
