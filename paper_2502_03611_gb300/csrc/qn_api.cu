@@ -623,6 +623,11 @@ extern "C" int qn_ctx_create(const qn_problem *p, qn_ctx **out) {
             (p->bc == QN_BC_DIRICHLET || p->bc == QN_BC_NEUMANN) && p->potential_host == nullptr) {
             CK(cudaMalloc(&c->small_bar, kSmallBarWords * sizeof(unsigned)));
             CK(cudaMemset(c->small_bar, 0, kSmallBarWords * sizeof(unsigned)));
+            rc = small_solve_set_attributes();
+            if (rc != QN_OK) {
+                ctx_free(c);
+                return rc;
+            }
             c->small_solve = 1;
         }
         // the closed-form sine / cosine pairs have the reflection symmetry the split

@@ -262,7 +262,7 @@ int launch_modeprod_tc_split(TcPlan *plan, int src, int dst, Epi epi, const EpiA
                              bool x6 = false);
 // ---- whole-solve persistent kernel for small 2-D FP64 problems (qn_small.cu) ----------
 constexpr int kSmallMaxN = 128;
-constexpr int kSmallBarWords = 64;   // the grid barrier's counter and generation words, apart
+constexpr int kSmallBarWords = 64 + kSmallMaxN;   // the barrier's counter and generation words, apart; row flags
 struct SmallSolve {
     double *U;
     const double *f;
@@ -280,6 +280,7 @@ struct SmallSolve {
     int beta_fixed, max_it;
 };
 int small_solve_supported(int dim, int n);
+int small_solve_set_attributes();   // once, before the first launch
 // One cooperative launch that runs the whole solve; on return (asynchronous) st holds
 // it / status / done as the finaliser leaves them, hist the per-iterate statistics.
 int launch_small_solve(const SmallSolve &q, cudaStream_t s);

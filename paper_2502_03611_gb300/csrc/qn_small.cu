@@ -2,28 +2,32 @@
 // with the inverse of Sec. 4.1 eq. fin_inverse), n <= kSmallMaxN.
 //
 // At these sizes every phase of an iteration is a few microseconds of work (the 63^2
-// grid has 3969 unknowns; one mode product is 250k FP64 FMAs), so a solve made of
+// grid has 3969 unknowns; one mode product is 125k FP64 FMAs), so a solve made of
 // separate launches is bound by launch and host-check latency. Here one cooperative
-// launch runs the whole solve, the phases separated by a grid barrier. Block b owns rows
-// b, b + grid, ... of every phase's input: it evaluates the residual on its rows of U, and
-// in a product stages its input row in shared memory and forms the n outputs that row
-// feeds (the matrix rows come from L1, where S and S^{-1} stay between iterations).
+// launch runs the whole solve; block b owns row y = b of the grid and mode kx = b (and
+// b + grid, ... with fewer blocks than rows).
 //
-//   iteration k:  residual r = A_h U + lam U + b U^3 - f  (+ block partials of ||r||^2,
-//                 ||f||^2 at k = 0, min / max U^2), and on the same rows
-//                 P1  Y1[kx][y] = sum_x S^{-1}[kx][x] r[y][x]              -> barrier
+//   iteration k:  wait for the neighbouring rows' updates (one flag word per row)
+//                 residual r = A_h U + lam U + b U^3 - f of the row (+ block partials of
+//                 ||r||^2, ||f||^2 at k = 0, min / max U^2), and from it
+//                 P1  Y1[kx][y] = sum_x S^{-1}[kx][x] r[y][x]          -> grid barrier
 //                 every block reduces the partial records in the same order, so all
 //                 take the same stop decision and the same beta_n = (min + max)/2 of
 //                 3 b U^2; block 0 records the iterate's statistics
-//                 P2  Y2[ky][kx] = sum_y S^{-1}[ky][y] Y1[kx][y] / (lam_kx + lam_ky + lam + beta_n)
-//                                                                           -> barrier
-//                 P3  Y3[x][ky] = sum_kx S[x][kx] Y2[ky][kx]               -> barrier
-//                 P4  U[y][x] -= step * sum_ky S[y][ky] Y3[x][ky]          -> barrier
+//                 P2  Y2[ky] = sum_y S^{-1}[ky][y] Y1[kx][y] / (lam_kx + lam_ky + lam + beta_n)
+//                 P3  Z[y][kx] = sum_ky S[y][ky] Y2[ky], in the same block  -> grid barrier
+//                 P4  U[y][x] -= step * sum_kx S[x][kx] Z[y][kx]; the row's flag
 //
-// Each product stores its output transposed, so every dot product reads two contiguous
-// rows. The barrier is a counter and a generation word in global memory; every wait is
-// bounded (2 s of %globaltimer), after which the block sets the error word, and all
-// blocks leave at their next barrier. The launch is cooperative, so all blocks are
+// The backward transform takes y first, so that a mode's column never leaves its block:
+// two grid barriers an iteration and a wait for two neighbours, where the order of the
+// large solves needs four barriers. The products use the reflection symmetry (half the
+// FP64 work, see qn_modeprod_f64tc.cu), with both half matrices transposed in shared
+// memory: read from L1 by rows, a warp's 32 lanes touched 32 lines for every term, and
+// the four products took most of an iteration. 273 -> 190 us per 63^2 solve of seven iterations
+// (the kernel 235 -> 140 us).
+//
+// Every wait is bounded (2 s of %globaltimer), after which the block sets the error word,
+// and all blocks leave at their next wait. The launch is cooperative, so all blocks are
 // resident at once.
 #include <math.h>
 #include <stdio.h>
@@ -38,6 +42,7 @@ namespace {
 
 constexpr int kSmallThreads = 128;
 constexpr int kBarGen = 32;   // the generation word, a 128-byte line away from the counter
+constexpr int kBarFlags = 64; // one word per row: updates applied to it
 constexpr unsigned long long kSmallTimeoutNs = 2000000000ull;
 
 __device__ __forceinline__ unsigned long long small_timer() {
@@ -92,7 +97,7 @@ struct SmallArgs {
     const double *S, *Si, *lam1;   // n x n row-major (S[:, k] eigenvector k), eigenvalues
     double *w0, *w1;               // n^2 work arrays
     double *partials;              // [gridDim][4]
-    unsigned *bar;                 // [2] barrier counter, generation
+    unsigned *bar;                 // barrier counter, generation, row flags
     DevState *st;                  // it / status / done on return
     qn_stats *hist;
     int hist_cap;
@@ -102,120 +107,173 @@ struct SmallArgs {
     int beta_fixed, max_it;
 };
 
-__device__ __forceinline__ double nb_value(const double *U, int x, int y, int n, bool neu) {
-    if (neu) {
-        x = (x == -1) ? 1 : (x == n ? n - 2 : x);
-        y = (y == -1) ? 1 : (y == n ? n - 2 : y);
-    }
-    return (x < 0 || x >= n || y < 0 || y >= n) ? 0.0 : __ldcg(U + y * n + x);
-}
-
-// One product phase: out[a][b] = sum_j M[a][j] X[b][j] (/ (lam_a + lam_b + shift) with a
-// divide) for the input rows b this block owns (b = blockIdx.x, + gridDim.x, ...). The
-// block stages its row of X (written by other blocks in the previous phase) in shared
-// memory, read through L2; M is read-only and stays in L1 from one iteration to the next.
-template <bool DIVIDE>
-__device__ __forceinline__ void small_product(const double *__restrict__ M, const double *X, double *out, int n,
-                                              double *row, const double *lam1, double shift) {
-    for (int b = blockIdx.x; b < n; b += gridDim.x) {
-        __syncthreads();
-        for (int j = threadIdx.x; j < n; j += blockDim.x) row[j] = __ldcg(X + b * n + j);
-        __syncthreads();
-        for (int a = threadIdx.x; a < n; a += blockDim.x) {
-            const double *m = M + a * n;
-            double s0 = 0.0, s1 = 0.0;
-            int j = 0;
-            for (; j + 2 <= n; j += 2) {
-                s0 = fma(__ldg(m + j), row[j], s0);
-                s1 = fma(__ldg(m + j + 1), row[j + 1], s1);
+// Wait (thread 0) until the two neighbouring rows of row y have had `it` updates.
+__device__ bool wait_rows(const unsigned *flags, int y, int n, unsigned it, int *err) {
+    for (int k = -1; k <= 1; k += 2) {
+        const int r = y + k;
+        if (r < 0 || r >= n) continue;
+        const unsigned long long t0 = small_timer();
+        unsigned polls = 0;
+        while (ld_acquire(flags + r) < it) {
+            if ((++polls & 63u) == 0 && (*(volatile int *)err != 0 || small_timer() - t0 > kSmallTimeoutNs)) {
+                atomicExch(err, QN_ETIMEOUT);
+                return false;
             }
-            if (j < n) s0 = fma(__ldg(m + j), row[j], s0);
-            double v = s0 + s1;
-            if (DIVIDE) v = v / ((__ldg(lam1 + b) + __ldg(lam1 + a)) + shift);
-            out[a * n + b] = v;
         }
     }
+    return true;
+}
+
+// Four chains of the terms 0 .. len - 1 of column t of a table with row stride n.
+__device__ __forceinline__ double dot_column(const double *tab, const double *v, int vs, int len, int n, int t) {
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+    int j = 0;
+    for (; j + 4 <= len; j += 4) {
+        s0 = fma(tab[j * n + t], v[j * vs], s0);
+        s1 = fma(tab[(j + 1) * n + t], v[(j + 1) * vs], s1);
+        s2 = fma(tab[(j + 2) * n + t], v[(j + 2) * vs], s2);
+        s3 = fma(tab[(j + 3) * n + t], v[(j + 3) * vs], s3);
+    }
+    for (; j < len; ++j) s0 = fma(tab[j * n + t], v[j * vs], s0);
+    return (s0 + s1) + (s2 + s3);
+}
+
+// Forward product of the row in v (n values, overwritten by its mirror sums and differences):
+// thread k < n returns sum_j S^{-1}[k][j] v[j].
+__device__ __forceinline__ double small_forward(const double *F, double *v, int n, int t) {
+    const int nsym = (n + 1) >> 1, nanti = n >> 1;
+    double x = 0.0, y = 0.0;
+    if (t < nsym) {
+        x = v[t];
+        y = (t < nanti) ? v[n - 1 - t] : 0.0;
+    }
+    __syncthreads();
+    if (t < nsym) v[t] = x + y;
+    if (t < nanti) v[nsym + t] = x - y;
+    __syncthreads();
+    if (t >= n) return 0.0;
+    // one loop for both parities (a branch would run them one after the other)
+    return dot_column(F, v + ((t & 1) ? nsym : 0), 1, (t & 1) ? nanti : nsym, n, t);
+}
+
+// Backward product of the modes in v: thread s < n returns sum_k S[s][k] v[k]. q: n doubles.
+__device__ __forceinline__ double small_backward(const double *B, const double *v, double *q, int n, int t) {
+    const int nsym = (n + 1) >> 1, nanti = n >> 1;
+    // p_t over the even modes, q_{t - nsym} over the odd ones
+    if (t < n) q[t] = dot_column(B, v + (t < nsym ? 0 : 1), 2, t < nsym ? nsym : nanti, n, t);
+    __syncthreads();
+    double d = 0.0;
+    if (t < nsym)
+        d = q[t] + (t < nanti ? q[nsym + t] : 0.0);
+    else if (t < n)
+        d = q[n - 1 - t] - q[nsym + (n - 1 - t)];
+    __syncthreads();
+    return d;
 }
 
 __global__ void __launch_bounds__(kSmallThreads) k_small2d_fp64(SmallArgs a) {
-    extern __shared__ double row[];   // one row of the phase input (n doubles)
-    __shared__ double red[4][kSmallThreads / 32];
+    // F[j][k] = S^{-1}[k][j], j < ceil(n/2); B[i][t] = S[t][2i] (t < ceil(n/2)), S[t - ceil(n/2)][2i+1];
+    // three rows of scratch; the block's rows of U
+    extern __shared__ double sm[];
     __shared__ double sh_beta, sh_fn;
-    __shared__ int sh_stop;
-    const int n = a.n;
+    __shared__ int sh_stop, sh_ok;
+    const int n = a.n, nsym = (n + 1) >> 1, nanti = n >> 1;
+    double *F = sm, *B = F + nsym * n, *row = B + nsym * n, *tmp = row + n, *rc = tmp + n, *Ur = rc + n;
     const bool neu = a.neumann != 0;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = threadIdx.x;
+    unsigned *flags = a.bar + kBarFlags;
+    for (int e = t; e < n * nsym; e += kSmallThreads) {
+        const int k = e / nsym, j = e - k * nsym;   // rows of the matrices: coalesced reads
+        F[j * n + k] = __ldg(a.Si + k * n + j);
+        const int sr = k < nsym ? k : k - nsym, md = k < nsym ? 2 * j : 2 * j + 1;
+        B[j * n + k] = md < n ? __ldg(a.S + sr * n + md) : 0.0;
+    }
+    {
+        int i = 0;
+        for (int y = blockIdx.x; y < n; y += gridDim.x, ++i)
+            for (int x = t; x < n; x += kSmallThreads) Ur[i * n + x] = __ldcg(a.U + y * n + x);
+    }
+    if (t == 0) sh_ok = 1;
+    __syncthreads();
     double fn = 0.0;
     int it = 0;
     int status = QN_ENOTCONV;
+    // The last warp has no outputs of a product up to n = 96: it takes the reductions and the
+    // stop decision while the others run the products.
+    constexpr int kRedWarp = kSmallThreads / 32 - 1;
     for (;; ++it) {
-        // ---- residual of the rows this block owns, and its partial record
+        // ---- residual of the rows this block owns, its partial record, and P1
         double r2 = 0.0, f2 = 0.0, mn = INFINITY, mx = 0.0;
-        for (int y = blockIdx.x; y < n; y += gridDim.x)
-            for (int x = threadIdx.x; x < n; x += blockDim.x) {
-                const int p = y * n + x;
-                const double u = __ldcg(a.U + p);
-                const double lap = ((4.0 * u - nb_value(a.U, x - 1, y, n, neu)) - nb_value(a.U, x + 1, y, n, neu)) -
-                                   (nb_value(a.U, x, y - 1, n, neu) + nb_value(a.U, x, y + 1, n, neu));
-                const double fv = __ldg(a.f + p);
-                double t = fma(a.b, (u * u) * u, -fv);
-                t = fma(a.lam, u, t);
-                const double r = fma(lap, a.inv_h2, t);
-                a.w0[p] = r;
-                r2 = fma(r, r, r2);
-                if (it == 0) f2 = fma(fv, fv, f2);
-                mn = fmin(mn, u * u);
-                mx = fmax(mx, u * u);
+        int i = 0;
+        for (int y = blockIdx.x; y < n; y += gridDim.x, ++i) {
+            if (it > 0 && t == 0 && !wait_rows(flags, y, n, (unsigned)it, a.err)) sh_ok = 0;
+            __syncthreads();
+            if (!sh_ok) return;
+            if (t < n) {
+                const double *ur = Ur + i * n;
+                const int yu = y > 0 ? y - 1 : (neu ? 1 : -1), yd = y < n - 1 ? y + 1 : (neu ? n - 2 : -1);
+                const double up = yu >= 0 ? __ldcg(a.U + yu * n + t) : 0.0;
+                const double dn = yd >= 0 ? __ldcg(a.U + yd * n + t) : 0.0;
+                const double le = t > 0 ? ur[t - 1] : (neu ? ur[1] : 0.0);
+                const double ri = t < n - 1 ? ur[t + 1] : (neu ? ur[n - 2] : 0.0);
+                const double u = ur[t];
+                const double lap = ((4.0 * u - le) - ri) - (up + dn);
+                const double fv = __ldg(a.f + y * n + t);
+                double v = fma(a.b, (u * u) * u, -fv);
+                v = fma(a.lam, u, v);
+                const double r = fma(lap, a.inv_h2, v);
+                row[t] = r;
+                rc[t] = r;
             }
-        for (int o = 16; o > 0; o >>= 1) {
-            r2 += __shfl_xor_sync(0xffffffffu, r2, o);
-            f2 += __shfl_xor_sync(0xffffffffu, f2, o);
-            mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-            mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            __syncthreads();
+            const double v = small_forward(F, row, n, t);
+            if (t < n) a.w1[t * n + y] = v;   // Y1[kx = t][y]
+            if (warp == kRedWarp)
+                for (int x = lane; x < n; x += 32) {
+                    const double r = rc[x], u = Ur[i * n + x], u2 = u * u;
+                    r2 = fma(r, r, r2);
+                    if (it == 0) {
+                        const double fv = __ldg(a.f + y * n + x);
+                        f2 = fma(fv, fv, f2);
+                    }
+                    mn = fmin(mn, u2);
+                    mx = fmax(mx, u2);
+                }
         }
-        if (lane == 0) {
-            red[0][warp] = r2;
-            red[1][warp] = f2;
-            red[2][warp] = mn;
-            red[3][warp] = mx;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double q0 = red[0][0], q1 = red[1][0], q2 = red[2][0], q3 = red[3][0];
-            for (int w = 1; w < kSmallThreads / 32; ++w) {
-                q0 += red[0][w];
-                q1 += red[1][w];
-                q2 = fmin(q2, red[2][w]);
-                q3 = fmax(q3, red[3][w]);
+        if (warp == kRedWarp) {
+            for (int o = 16; o > 0; o >>= 1) {
+                r2 += __shfl_xor_sync(0xffffffffu, r2, o);
+                if (it == 0) f2 += __shfl_xor_sync(0xffffffffu, f2, o);
+                mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+                mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
             }
-            double *q = a.partials + 4 * blockIdx.x;
-            q[0] = q0;
-            q[1] = q1;
-            q[2] = q2;
-            q[3] = q3;
+            if (lane == 0) {
+                double *q = a.partials + 4 * blockIdx.x;
+                q[0] = r2;
+                q[1] = f2;
+                q[2] = mn;
+                q[3] = mx;
+            }
         }
-        // P1  Y1[kx][y] = sum_x Si[kx][x] r[y][x] on the rows just evaluated (this block's
-        // own), before the barrier: it needs neither the norms nor beta
-        small_product<false>(a.Si, a.w0, a.w1, n, row, nullptr, 0.0);
         if (!small_barrier(a.bar, a.bar + kBarGen, a.err)) return;
         // ---- every block: the same reduction, the same decision
-        if (warp == 0) {
-            double R = 0.0, F = 0.0, MN = INFINITY, MX = 0.0;
+        auto decide = [&]() {
+            double R = 0.0, F2 = 0.0, MN = INFINITY, MX = 0.0;
             for (int i = lane; i < (int)gridDim.x; i += 32) {
                 const double *q = a.partials + 4 * i;
                 R += __ldcg(q + 0);
-                F += __ldcg(q + 1);
+                F2 += __ldcg(q + 1);
                 MN = fmin(MN, __ldcg(q + 2));
                 MX = fmax(MX, __ldcg(q + 3));
             }
             for (int o = 16; o > 0; o >>= 1) {
                 R += __shfl_xor_sync(0xffffffffu, R, o);
-                F += __shfl_xor_sync(0xffffffffu, F, o);
+                F2 += __shfl_xor_sync(0xffffffffu, F2, o);
                 MN = fmin(MN, __shfl_xor_sync(0xffffffffu, MN, o));
                 MX = fmax(MX, __shfl_xor_sync(0xffffffffu, MX, o));
             }
             if (lane == 0) {
-                if (it == 0) sh_fn = sqrt(F);
+                if (it == 0) sh_fn = sqrt(F2);
                 const double res = sqrt(R);
                 const double f_norm = sh_fn;
                 const double fa = 3.0 * a.b * MN, fb = 3.0 * a.b * MX;
@@ -247,40 +305,47 @@ __global__ void __launch_bounds__(kSmallThreads) k_small2d_fp64(SmallArgs a) {
                 sh_stop = stop;
                 sh_beta = a.lam + beta;
             }
-        }
-        __syncthreads();
-        fn = sh_fn;
-        if (sh_stop) break;
-        const double shift = sh_beta;
-        // P2  Y2[ky][kx] = sum_y Si[ky][y] Y1[kx][y] / (lam_kx + lam_ky + shift)
-        small_product<true>(a.Si, a.w1, a.w0, n, row, a.lam1, shift);
-        if (!small_barrier(a.bar, a.bar + kBarGen, a.err)) return;
-        // P3  Y3[x][ky] = sum_kx S[x][kx] Y2[ky][kx]
-        small_product<false>(a.S, a.w0, a.w1, n, row, nullptr, 0.0);
-        if (!small_barrier(a.bar, a.bar + kBarGen, a.err)) return;
-        // P4  delta[y][x] = sum_ky S[y][ky] Y3[x][ky], U -= step * delta
-        for (int b = blockIdx.x; b < n; b += gridDim.x) {   // b = x (the input row)
+        };
+        // P2, P3 of the modes kx this block owns; the decision falls during the first P2
+        bool stop = false;
+        for (int kx = blockIdx.x; kx < n; kx += gridDim.x) {
             __syncthreads();
-            for (int j = threadIdx.x; j < n; j += blockDim.x) row[j] = __ldcg(a.w1 + b * n + j);
+            if (t < n) row[t] = __ldcg(a.w1 + kx * n + t);
             __syncthreads();
-            for (int y = threadIdx.x; y < n; y += blockDim.x) {
-                const double *m = a.S + y * n;
-                double s0 = 0.0, s1 = 0.0;
-                int j = 0;
-                for (; j + 2 <= n; j += 2) {
-                    s0 = fma(__ldg(m + j), row[j], s0);
-                    s1 = fma(__ldg(m + j + 1), row[j + 1], s1);
-                }
-                if (j < n) s0 = fma(__ldg(m + j), row[j], s0);
-                const double d = s0 + s1;
-                const int p = y * n + b;
-                const double u = __ldcg(a.U + p);
-                a.U[p] = (a.step == 1.0) ? u - d : fma(-a.step, d, u);
+            double v = small_forward(F, row, n, t);
+            if (kx == (int)blockIdx.x) {
+                if (warp == kRedWarp) decide();
+                __syncthreads();
+                fn = sh_fn;
+                stop = sh_stop != 0;
+                if (stop) break;
             }
+            const double shift = sh_beta;
+            if (t < n) tmp[t] = v / ((__ldg(a.lam1 + kx) + __ldg(a.lam1 + t)) + shift);
+            __syncthreads();
+            v = small_backward(B, tmp, row, n, t);
+            if (t < n) a.w0[t * n + kx] = v;   // Z[y = t][kx]
         }
+        if (stop) break;
         if (!small_barrier(a.bar, a.bar + kBarGen, a.err)) return;
+        // P4 and the update of the rows
+        i = 0;
+        for (int y = blockIdx.x; y < n; y += gridDim.x, ++i) {
+            if (t < n) tmp[t] = __ldcg(a.w0 + y * n + t);
+            __syncthreads();
+            const double d = small_backward(B, tmp, row, n, t);
+            if (t < n) {
+                const double u = Ur[i * n + t];
+                const double w = (a.step == 1.0) ? u - d : fma(-a.step, d, u);
+                Ur[i * n + t] = w;
+                a.U[y * n + t] = w;
+            }
+            __syncthreads();
+            if (t == 0)
+                asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(flags + y), "r"((unsigned)(it + 1)) : "memory");
+        }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 32 * kRedWarp) {   // the lane that decided
         a.st->it = it;
         a.st->status = status;
         a.st->done = 1;
@@ -292,31 +357,32 @@ __global__ void __launch_bounds__(kSmallThreads) k_small2d_fp64(SmallArgs a) {
 
 int small_solve_supported(int dim, int n) { return dim == 2 && n >= 1 && n <= kSmallMaxN; }
 
+// Shared memory for `grid` blocks: both half matrices, three rows of scratch, the block's rows.
+static size_t small_smem(int n, int grid) {
+    const int nsym = (n + 1) / 2, rows = (n + grid - 1) / grid;
+    return sizeof(double) * ((size_t)2 * nsym * n + 3 * n + (size_t)rows * n);
+}
+
+int small_solve_set_attributes() {
+    QN_CUDA(cudaFuncSetAttribute(k_small2d_fp64, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+    return QN_OK;
+}
+
 int launch_small_solve(const SmallSolve &q, cudaStream_t s) {
-    static int blocks_per_sm = -1;
-    if (blocks_per_sm < 0) {
-        int nb = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_small2d_fp64, kSmallThreads,
-                                                          sizeof(double) * kSmallMaxN) != cudaSuccess)
-            nb = 0;
-        blocks_per_sm = nb;
-    }
-    if (blocks_per_sm < 1) {
-        set_error("launch_small_solve: the kernel does not fit on an SM");
-        return QN_ECUDA;
-    }
     // one block per SM (the phases are FP64-FMA bound: about 2 FMAs per clock per SM on
-    // this GPU), never more blocks than points
-    // one block per row of the phase inputs (each block owns rows b, b + grid, ...)
+    // this GPU) and per row
     const char *eg = getenv("QN_SMALL_GRID");
     int grid = eg ? atoi(eg) : q.n;
     if (grid > q.num_sms) grid = q.num_sms;
     if (grid > q.n) grid = q.n;
     if (grid < 1) grid = 1;
-    const int cap = blocks_per_sm * q.num_sms;
-    if (grid > cap) grid = cap;
     if (grid > q.partials_cap) grid = q.partials_cap;
     if (grid < 1) grid = 1;
+    if (small_smem(q.n, grid) > 220 * 1024) {
+        set_error("launch_small_solve: %d rows of n = %d per block do not fit in shared memory", (q.n + grid - 1) / grid,
+                  q.n);
+        return QN_EINVAL;
+    }
     SmallArgs a;
     a.U = q.U;
     a.f = q.f;
@@ -344,7 +410,7 @@ int launch_small_solve(const SmallSolve &q, cudaStream_t s) {
     QN_CUDA(cudaMemsetAsync(q.bar, 0, kSmallBarWords * sizeof(unsigned), s));
     void *params[] = {&a};
     QN_CUDA(cudaLaunchCooperativeKernel((const void *)k_small2d_fp64, dim3(grid), dim3(kSmallThreads), params,
-                                        sizeof(double) * q.n, s));
+                                        small_smem(q.n, grid), s));
     return QN_OK;
 }
 
