@@ -119,7 +119,7 @@ struct qn_ctx {
     cudaEvent_t hm_in_ready[2], hm_solved[2], hm_out_done[2];
     float *warm_dsq;      // device: ||U_1 - U_0||^2 of a warm-started solve's first iteration
     int warm_dsq_on;      // 1 while that iteration's products are enqueued
-    // reflection-split mode products (3-D split solve, P a multiple of 128)
+    // reflection-split mode products (3-D split solve, tc_split_sizes)
     int split;            // 1: the plan holds the split matrices and the solve loop uses them
     int split_layout;     // 1: the last residual wrote its planes in split / folded order
     int last_split;       // 1: the last shifted inverse used the split products
@@ -701,7 +701,7 @@ extern "C" int qn_ctx_create(const qn_problem *p, qn_ctx **out) {
         // S^{-1}[k][n-1-j] = (-1)^k S^{-1}[k][j].
         const char *es = getenv("QN_SPLIT");
         const bool want_split = es ? (atoi(es) != 0) : true;
-        if (want_split && c->dim == 3 && P % 128 == 0 && c->fdf != nullptr) {
+        if (want_split && c->dim == 3 && tc_split_sizes(P) && c->fdf != nullptr) {
             const int H = P / 2, nsym = (n + 1) / 2, nanti = n / 2;
             std::vector<__nv_bfloat16> fh((size_t)P * H), fl((size_t)P * H), bh((size_t)P * H), blo((size_t)P * H);
             std::vector<float> ls(P, 1e30f);
@@ -741,7 +741,7 @@ extern "C" int qn_ctx_create(const qn_problem *p, qn_ctx **out) {
                 ctx_free(c);
                 return rc;
             }
-            if (c->split) {
+            if (c->split && P % 128 == 0) {
                 // third level of the backward matrix (after the hi / lo above; small, kept for
                 // qn_ctx_set_escalation too); the working buffers' level only for BF16X6
                 std::vector<__nv_bfloat16> bl2v((size_t)P * H);
@@ -756,7 +756,7 @@ extern "C" int qn_ctx_create(const qn_problem *p, qn_ctx **out) {
                 CK(cudaMalloc(&c->bb_l2, bb));
                 CK(cudaMemcpy(c->bb_l2, bl2v.data(), bb, cudaMemcpyHostToDevice));
             }
-            if (c->split && want_x6) {
+            if (c->bb_l2 != nullptr && want_x6) {
                 rc = ensure_x6(c);
                 if (rc != QN_OK) {
                     ctx_free(c);
@@ -1202,8 +1202,9 @@ extern "C" int qn_set_escalation(qn_ctx *c, double rate) {
         return QN_EINVAL;
     }
     if (rate > 0.0 && c->x6_base == 0) {
-        if (c->prob.precision != QN_PREC_BF16X3 || !c->split) {
-            set_error("qn_set_escalation: needs a BF16X3 context with the reflection-split products");
+        if (c->prob.precision != QN_PREC_BF16X3 || c->bb_l2 == nullptr) {
+            set_error("qn_set_escalation: needs a BF16X3 context with the reflection-split products and P a "
+                      "multiple of 128");
             return QN_EUNSUPPORTED;
         }
         rc = ensure_x6(c);
@@ -1224,7 +1225,8 @@ extern "C" int qn_set_fused_residual(qn_ctx *c, int on) {
             return QN_EUNSUPPORTED;
         }
         rc = tc_plan_enable_fused(c->plan);
-        if (rc == QN_EUNSUPPORTED) set_error("qn_set_fused_residual: the fused kernel takes P <= 512");
+        if (rc == QN_EUNSUPPORTED)
+            set_error("qn_set_fused_residual: the fused kernel takes P <= 512, a multiple of 128");
         if (rc) return rc;
     }
     c->fused = on ? 1 : 0;

@@ -262,7 +262,7 @@ __device__ __forceinline__ double eig_point(double *__restrict__ U, const double
 
 // U = s U~, F into the inverse's input, per-block sum of w F^2 (times h^dim) and the
 // extremes of lam + 3 b U^2 + V. OUT 0: FP64 n^DIM array. OUT 1: BF16 hi/lo planes on
-// the padded P^DIM grid in natural order. OUT 2 (3-D, P a multiple of 128): the
+// the padded P^DIM grid in natural order. OUT 2 (3-D, tc_split_sizes): the
 // reflection-split order of k_residual_mirror (x: sums at i, differences at P/2 + i;
 // y, z folded).
 template <int DIM, int OUT, bool NEU>
@@ -778,8 +778,8 @@ int launch_eig_pass2(double *U, const double *lin, int n, int P, int dim, int bc
         else
             pass2_t<2, 0>(U, lin, n, P, neu, hd, lam, b, pot, R64, Rhi, Rlo, partials, grid, st, s);
     } else if (mirror) {
-        if (dim != 3 || P % 128 != 0) {
-            set_error("launch_eig_pass2: the reflection-split layout needs 3-D and P a multiple of 128");
+        if (dim != 3 || !tc_split_sizes(P)) {
+            set_error("launch_eig_pass2: the reflection-split layout needs 3-D and a size of the split products");
             return QN_EINVAL;
         }
         pass2_t<3, 2>(U, lin, n, P, neu, hd, lam, b, pot, R64, Rhi, Rlo, partials, grid, st, s);
@@ -885,8 +885,8 @@ int launch_eig_pass2_df(double *U, const float2 *lin, int n, int P, int dim, int
     const bool neu = (bc == QN_BC_NEUMANN);
     int rc;
     if (mirror) {
-        if (dim != 3 || P % 128 != 0) {
-            set_error("launch_eig_pass2_df: the reflection-split layout needs 3-D and P a multiple of 128");
+        if (dim != 3 || !tc_split_sizes(P)) {
+            set_error("launch_eig_pass2_df: the reflection-split layout needs 3-D and a size of the split products");
             return QN_EINVAL;
         }
         rc = pass2_df_t<3, 2>(U, lin, n, P, neu, hd, lam, b, pot32, Rhi, Rlo, partials, grid, used, st, s);

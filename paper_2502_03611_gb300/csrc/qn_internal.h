@@ -244,7 +244,12 @@ void tc_plan_destroy(TcPlan *plan);
 // the FP64 dense target for EPI_UPDATE / EPI_DENSE). forward selects S^{-1}.
 int launch_modeprod_tc(TcPlan *plan, int src, int dst, bool forward, Epi epi,
                        const EpiArgs &e, cudaStream_t s);
-// Reflection-split products (3-D, P a multiple of 128): B_fwd, B_bwd are the
+// Sizes the reflection-split products are used at (3-D). P = 192 is left to the dense products: a
+// solve takes 1.34 ms against 1.45 at n = 130 and 1.57 against 1.72 at n = 192, the halves of 96
+// filling the MMAs too little; from P = 320 on the split is faster (5.9 against 5.0 ms at n = 260,
+// 14.4 against 13.1 at 400, 50.7 against 43.0 at 640, 161 against 119 at 850; 8 iterations each).
+inline bool tc_split_sizes(int P) { return P % 128 == 0 || (P % 64 == 0 && P >= 320); }
+// Reflection-split products (3-D): B_fwd, B_bwd are the
 // [P][P/2] split-precision matrices described in qn_modeprod_tc.cu. Returns
 // QN_EUNSUPPORTED when the sizes do not allow it (the plan keeps the dense path).
 int tc_plan_enable_split(TcPlan *plan, const __nv_bfloat16 *bf_hi, const __nv_bfloat16 *bf_lo,

@@ -26,8 +26,7 @@
 // S stays resident in L2). The epilogue of tile i overlaps the MMAs of tile
 // i+1 through the double-buffered accumulators.
 //
-// Reflection-split products (MODE 1 and 2; 3-D split solve with P a multiple
-// of 128, H = P/2). The sine basis satisfies S[n-1-j][k] = (-1)^k S[j][k], so
+// Reflection-split products (MODE 1 and 2; 3-D split solve, H = P/2; tc_split_sizes). The sine basis satisfies S[n-1-j][k] = (-1)^k S[j][k], so
 // along one axis
 //   forward:  Xhat[2i]   = sum_j S[j][2i]   a_j,  a_j = x_j + x_{n-1-j} (+ the middle x of odd n)
 //             Xhat[2i+1] = sum_j S[j][2i+1] b_j,  b_j = x_j - x_{n-1-j}
@@ -235,7 +234,7 @@ __global__ void __maxnreg__(104)
             tile_info(t, g0, groups, tiles, G, m0, n0);
             if (group_done(G)) continue;
             const uint32_t tx_bytes = kLv * (a_bytes + (uint32_t)G.BN * kRowBytes);
-            const int Hh = G.P >> 1, KBh = Hh / BK;
+            const int Hh = G.P >> 1, KBh = (Hh + BK - 1) / BK;
             const int KB = (MODE == 0) ? G.P / BK : (MODE == 1 ? KBh : 2 * KBh);
             for (int kb = 0; kb < KB; ++kb) {
                 if (!wait_bar(empty_bar(s), ph ^ 1u, abort_flag, err)) {
@@ -288,7 +287,7 @@ __global__ void __maxnreg__(104)
             tile_info(t, g0, groups, tiles, G, m0, n0);
             if (group_done(G)) continue;
             const uint32_t idesc = ptx::idesc_bf16_f32(BM, (uint32_t)G.BN);
-            const int KBh = (G.P >> 1) / BK;
+            const int Hh = G.P >> 1, KBh = (Hh + BK - 1) / BK;
             const int KB = (MODE == 0) ? G.P / BK : (MODE == 1 ? KBh : 2 * KBh);
             if (!wait_bar(tempty_bar(acc), aph ^ 1u, abort_flag, err)) break;
             ptx::tc_fence_after();
@@ -297,14 +296,16 @@ __global__ void __maxnreg__(104)
                 const bool second = (MODE == 2) && kb >= KBh;
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN_MAX + (second ? G.BN : 0));
                 const int kb0 = second ? kb - KBh : kb;
+                // the last K step of a half is 32 columns where H is not a multiple of BK; the
+                // rest of its tiles (the other half's columns, zeros past the end) is not used
+                const int nk = (MODE == 0) ? kKSteps : min(BK, Hh - kb0 * BK) / 16;
                 if (!wait_bar(full_bar(s), ph, abort_flag, err)) {
                     ok = false;
                     break;
                 }
                 ptx::tc_fence_after();
                 const uint32_t st = base + (uint32_t)s * stage_bytes;
-#pragma unroll
-                for (int kk = 0; kk < kKSteps; ++kk) {
+                auto mma_step = [&](int kk) {
                     const uint32_t koff = (uint32_t)kk * 32u;
                     const uint64_t a_hi = ptx::smem_desc_kmajor(st + koff, kRowBytes, kLayout);
                     const uint64_t a_lo = ptx::smem_desc_kmajor(st + a_bytes + koff, kRowBytes, kLayout);
@@ -323,6 +324,12 @@ __global__ void __maxnreg__(104)
                         ptx::mma_bf16(d_tmem, a_hi, b_l2, idesc, 1u);
                         ptx::mma_bf16(d_tmem, a_l2, b_hi, idesc, 1u);
                     }
+                };
+                if (MODE == 0 || nk == kKSteps) {
+#pragma unroll
+                    for (int kk = 0; kk < kKSteps; ++kk) mma_step(kk);
+                } else {
+                    for (int kk = 0; kk < nk; ++kk) mma_step(kk);
                 }
                 ptx::mma_commit(empty_bar(s));
                 if (++s == stages) {
@@ -377,8 +384,10 @@ __global__ void __maxnreg__(104)
             const int kstride = (DIM == 3) ? n * n : n;
             const float dscale = G.dscale;
             const float step = G.step;
-            const int cols = BN / kEpiParts;   // >= 16: BN is 64, 128 or 256
+            // a multiple of 4 (BN is one of 16), in chunks of 16 with a shorter last one
+            const int cols = BN / kEpiParts;
             const int cbeg = part * cols, cend = cbeg + cols;
+            const int kend = min(P, n0 + cend);   // first output row past this warp's columns
             float dsq_acc = 0.0f;   // sum of squared updates (G.dsq)
             const int Hh = P >> 1;
             const int nsym = (n + 1) >> 1, nanti = n >> 1;
@@ -402,13 +411,14 @@ __global__ void __maxnreg__(104)
                         const float v = __uint_as_float(r[i]);
                         const float pv = __shfl_xor_sync(0xffffffffu, v, 1);
                         const float o = valid ? (odd ? pv - v : v + pv) : 0.0f;
-                        if (k0 + i < P) split_store(o, G.out_hi, G.out_lo, (k0 + i) * Mtot + obase);
+                        if (k0 + i < kend) split_store(o, G.out_hi, G.out_lo, (k0 + i) * Mtot + obase);
                     }
                 }
             }
             if (EPI == EPI_STORE_PQ) {
                 // p in columns [0, BN), q in [BN, 2 BN) of the accumulator; output
                 // rows j (< H) and n-1-j; the middle row of an odd n takes p alone
+                const int jsym = min(nsym, kend), janti = min(nanti, kend);   // this warp's rows
                 for (int c = cbeg; c < cend; c += kChunk) {
                     uint32_t rp[kChunk], rq[kChunk];
                     ptx::tmem_ld_32x32b_x16(tacc + (uint32_t)c, rp);
@@ -418,13 +428,12 @@ __global__ void __maxnreg__(104)
                     const int j0 = n0 + c;
 #pragma unroll
                     for (int i = 0; i < kChunk; ++i) {
-                        if (c + i >= cend) break;   // BN2/kEpiParts may be 24 (P = 384): half a chunk
                         const int j = j0 + i;
                         const float p = __uint_as_float(rp[i]), qv = __uint_as_float(rq[i]);
-                        if (j < nanti) {
+                        if (j < janti) {
                             store_lv<L3>(p + qv, G, l3, j * Mtot + m);
                             store_lv<L3>(p - qv, G, l3, (n - 1 - j) * Mtot + m);
-                        } else if (j < nsym) {
+                        } else if (j < jsym) {
                             store_lv<L3>(p, G, l3, j * Mtot + m);
                         }
                     }
@@ -441,25 +450,26 @@ __global__ void __maxnreg__(104)
                     if (!m_ok) continue;
                     const int j0 = n0 + c;
                     if (ubase >= 0) {
+                        const int jsym = min(nsym, kend), janti = min(nanti, kend);   // this warp's rows
                         double *ub = G.U + ubase;
                         double oa[8], ob[8];
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             const int j = j0 + i;
-                            oa[i] = (j < nsym) ? ub[j * kstride] : 0.0;
-                            ob[i] = (j < nanti) ? ub[(n - 1 - j) * kstride] : 0.0;
+                            oa[i] = (j < jsym) ? ub[j * kstride] : 0.0;
+                            ob[i] = (j < janti) ? ub[(n - 1 - j) * kstride] : 0.0;
                         }
                         const double st = (double)step;
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             const int j = j0 + i;
                             const float p = __uint_as_float(rp[i]), qv = __uint_as_float(rq[i]);
-                            const float xa = (j < nanti) ? p + qv : p, xb = p - qv;
-                            if (j < nsym) dsq_acc = fmaf(xa, xa, dsq_acc);
-                            if (j < nanti) dsq_acc = fmaf(xb, xb, dsq_acc);
-                            if (j < nsym)
+                            const float xa = (j < janti) ? p + qv : p, xb = p - qv;
+                            if (j < jsym) dsq_acc = fmaf(xa, xa, dsq_acc);
+                            if (j < janti) dsq_acc = fmaf(xb, xb, dsq_acc);
+                            if (j < jsym)
                                 ub[j * kstride] = (step == 1.0f) ? oa[i] - f2d_exact(xa) : fma(-st, f2d_exact(xa), oa[i]);
-                            if (j < nanti)
+                            if (j < janti)
                                 ub[(n - 1 - j) * kstride] =
                                     (step == 1.0f) ? ob[i] - f2d_exact(xb) : fma(-st, f2d_exact(xb), ob[i]);
                         }
@@ -475,12 +485,12 @@ __global__ void __maxnreg__(104)
                 if (EPI == EPI_STORE) {
 #pragma unroll
                     for (int i = 0; i < kChunk; ++i)
-                        if (k0 + i < P) split_store(__uint_as_float(r[i]), G.out_hi, G.out_lo, (k0 + i) * Mtot + m);
+                        if (k0 + i < kend) split_store(__uint_as_float(r[i]), G.out_hi, G.out_lo, (k0 + i) * Mtot + m);
                 } else if (EPI == EPI_DIVIDE) {
 #pragma unroll
                     for (int i = 0; i < kChunk; ++i) {
                         const int k = k0 + i;
-                        if (k < P) {
+                        if (k < kend) {
                             const float den = dscale * (__ldg(G.lam32 + k) + rowlam) + shift;
                             store_lv<L3>(__fdividef(__uint_as_float(r[i]), den), G, l3, k * Mtot + m);
                         }
@@ -689,24 +699,16 @@ int tc_plan_create(TcPlan **out, int n, int P, int dim, __nv_bfloat16 *bufs_hi[2
 int tc_plan_enable_split(TcPlan *p, const __nv_bfloat16 *bf_hi, const __nv_bfloat16 *bf_lo,
                          const __nv_bfloat16 *bb_hi, const __nv_bfloat16 *bb_lo) {
     const int H = p->P / 2;
-    if (p->dim != 3 || p->P % 128 != 0) return QN_EUNSUPPORTED;
-    // tile widths must divide H (a forward tile stays inside one half; the
-    // backward tiles cover the H rows exactly) and give every epilogue warp a
-    // whole number of TMEM chunks: BN1/kEpiParts a multiple of kChunk (16),
-    // BN2/kEpiParts a multiple of 8; BN2 <= 128 (two accumulators per tile)
-    p->BN1 = 0;
-    for (int bn = BN_MAX; bn >= 16 * kEpiParts; bn -= 16 * kEpiParts)
-        if (H % bn == 0) {
-            p->BN1 = bn;
-            break;
-        }
-    p->BN2 = 0;
-    for (int bn = 128; bn >= 8 * kEpiParts; bn -= 8 * kEpiParts)
-        if (H % bn == 0) {
-            p->BN2 = bn;
-            break;
-        }
-    if (p->BN1 == 0 || p->BN2 == 0) return QN_EUNSUPPORTED;
+    if (p->dim != 3 || !tc_split_sizes(p->P)) return QN_EUNSUPPORTED;
+    // The fewest tiles that cover a half, as even as 16 columns allow (the widest multiple of
+    // 32 that divides H = 320 or 448 is 64, whose tiles read A seven times at H = 448). Forward
+    // tiles stay inside a half (their BN1 divides H: 64 to 256 for every P to 1024); the rows of a
+    // backward tile past H are the other half's and are not stored. BN2 <= 128: two
+    // accumulators per tile.
+    const int t1 = (H + BN_MAX - 1) / BN_MAX, t2 = (H + 127) / 128;
+    p->BN1 = H / t1;
+    p->BN2 = ((H + t2 - 1) / t2 + 15) / 16 * 16;
+    if (p->BN1 * t1 != H || p->BN1 % 16 != 0) return QN_EUNSUPPORTED;
     CUtensorMap h[4];
     int rc = tc_encode_2d(&h[0], bf_hi, H, p->P, p->BK, p->BN1, p->BK);
     if (rc == QN_OK) rc = tc_encode_2d(&h[1], bf_lo, H, p->P, p->BK, p->BN1, p->BK);
@@ -721,7 +723,7 @@ int tc_plan_enable_split(TcPlan *p, const __nv_bfloat16 *bf_hi, const __nv_bfloa
 }
 
 int tc_plan_enable_fused(TcPlan *p) {
-    if (p == nullptr || !p->split || p->P > 512) return QN_EUNSUPPORTED;
+    if (p == nullptr || !p->split || p->P > 512 || p->P % 128 != 0) return QN_EUNSUPPORTED;
     if (p->fused) return QN_OK;
     const int H = p->P / 2;
     CUtensorMap h[2];
@@ -909,7 +911,7 @@ int launch_modeprod_tc_split(TcPlan *p, int src, int dst, Epi epi, const EpiArgs
     g.P = p->P;
     g.n = p->n;
     g.BN = fwd ? p->BN1 : p->BN2;
-    g.ntile_n = fwd ? p->P / p->BN1 : (p->P / 2) / p->BN2;
+    g.ntile_n = fwd ? p->P / p->BN1 : (p->P / 2 + p->BN2 - 1) / p->BN2;
     g.ntiles = g.ntile_n * (p->Mtot / BM);
     const int grid = g.ntiles < p->num_sms ? g.ntiles : p->num_sms;
     return p->BK == 64 ? split_launch<64>(p, g, l3, epi, x6, e.err, grid, s)

@@ -1861,9 +1861,9 @@ static int launch_mirror_kind(const ResidualArgs &a, int max_grid, int zchunk, i
 }
 
 int launch_residual_mirror(const ResidualArgs &a, int max_grid, int zchunk, int *grid_used, cudaStream_t s) {
-    if (a.dim != 3 || a.Rhi == nullptr || a.fdf == nullptr || a.fx_e == nullptr || a.P % 128 != 0 ||
+    if (a.dim != 3 || a.Rhi == nullptr || a.fdf == nullptr || a.fx_e == nullptr || !tc_split_sizes(a.P) ||
         zchunk < 1) {
-        set_error("launch_residual_mirror: needs a 3-D split residual, P a multiple of 128, the f copy");
+        set_error("launch_residual_mirror: needs a 3-D split residual at a size of the split products, the f copy");
         return QN_EINVAL;
     }
     if (a.pot != nullptr) {
