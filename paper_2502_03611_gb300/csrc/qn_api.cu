@@ -86,7 +86,7 @@ struct qn_ctx {
     int res_fp64_warps;   // residual inside the split solve: FP64-stencil warps per block (of 8)
     float2 *fdf;          // 3-D split solve: padded FP32-pair copy of f (k_residual_tiled)
     int res_tiled;        // 1: iterations >= 2 of a 3-D split solve use k_residual_tiled
-    int res_zc;           // planes per work item of k_residual_tiled
+    int res_zc;           // planes per work item of k_residual_tiled (0: chosen from the sizes)
     int res_parts;        // partial-sum records written by the last residual launch
     int res_fx_headroom;  // DevState::fx_headroom for the solves of this context
     int res_saved_fnorm;  // 1: the last residual's finaliser takes ||f|| from DevState::f_norm
@@ -478,8 +478,8 @@ extern "C" int qn_ctx_create(const qn_problem *p, qn_ctx **out) {
         const char *et = getenv("QN_RES_TILED");
         c->res_tiled = et ? (atoi(et) != 0) : 1;
         const char *ez = getenv("QN_RES_ZC");
-        const int zc = ez ? atoi(ez) : 32;
-        c->res_zc = (zc >= 1 && zc <= 4096) ? zc : 32;
+        const int zc = ez ? atoi(ez) : 0;
+        c->res_zc = (zc >= 1 && zc <= 4096) ? zc : 0;
         // exponent headroom of the fixed-point stencil (2 = room for 4x growth of
         // max|U|); smaller values route more planes through the exact path
         const char *eh = getenv("QN_RES_FX_HEADROOM");

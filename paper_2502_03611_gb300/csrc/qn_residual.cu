@@ -13,6 +13,7 @@
 // Per-block partials go to a fixed-size array; a one-block finaliser reduces
 // them in a fixed order (deterministic) and decides beta_n and convergence on
 // the device.
+#include <limits.h>
 #include <math.h>
 #include <string.h>
 
@@ -692,6 +693,37 @@ __device__ __forceinline__ void tile_partials(const ResidualArgs &a, float kr2, 
     }
 }
 
+// Zeros in the part of the padded planes that no tile with grid points covers: planes [n, P),
+// rows [yt, P) of the other planes, and `segs` segments of each other row from x = xt on, seg
+// elements apart and long up to the next one's start. Sixteen bytes per store (P is a multiple
+// of 64, xt, yt and seg of 16).
+__device__ __forceinline__ void zero_padding(const ResidualArgs &a, int xt, int yt, int seg, int segs) {
+    const unsigned n = a.n, P = a.P;
+    const unsigned tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    uint4 *hi = reinterpret_cast<uint4 *>(a.Rhi), *lo = reinterpret_cast<uint4 *>(a.Rlo);
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    const size_t plane = (size_t)P * P / 8, row = P / 8;
+    for (size_t i = tid; i < (P - n) * plane; i += nt) {
+        hi[n * plane + i] = zero;
+        lo[n * plane + i] = zero;
+    }
+    const unsigned c2 = (P - yt) * (unsigned)row;
+    for (size_t i = tid; i < (size_t)n * c2; i += nt) {
+        const size_t z = i / c2, o = z * plane + yt * row + (i - z * c2);
+        hi[o] = zero;
+        lo[o] = zero;
+    }
+    const unsigned w = (unsigned)(seg - xt) / 8, c3 = w * (unsigned)segs;
+    if (c3 == 0) return;
+    for (size_t i = tid; i < (size_t)n * yt * c3; i += nt) {
+        const unsigned r = (unsigned)(i / c3), k = (unsigned)(i - (size_t)r * c3);
+        const unsigned z = r / yt, y = r - z * yt;
+        const size_t o = z * plane + y * row + (k / w) * (unsigned)(seg / 8) + xt / 8 + k % w;
+        hi[o] = zero;
+        lo[o] = zero;
+    }
+}
+
 template <int KIND>
 __global__ void __launch_bounds__(kTThreads, 2) k_residual_tiled(ResidualArgs a, int zchunk) {
     if (a.done != nullptr && *(volatile const int *)a.done) return;
@@ -715,8 +747,8 @@ __global__ void __launch_bounds__(kTThreads, 2) k_residual_tiled(ResidualArgs a,
     const bool neu = (a.bc == QN_BC_NEUMANN);
     float dmn = INFINITY, dmx = -INFINITY;   // KIND 3: extremes of 3 b u^2 + V
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int tiles_x = P / kTX, tiles_y = P / kTY;
-    const int nzc = (P + zchunk - 1) / zchunk;
+    const int tiles_x = (n + kTX - 1) / kTX, tiles_y = (n + kTY - 1) / kTY;   // tiles with grid points
+    const int nzc = (n + zchunk - 1) / zchunk;
     const long long items = (long long)tiles_x * tiles_y * nzc;
     const long long nn = (long long)n * n;
     const unsigned long long *Ub = reinterpret_cast<const unsigned long long *>(a.U);
@@ -736,20 +768,9 @@ __global__ void __launch_bounds__(kTThreads, 2) k_residual_tiled(ResidualArgs a,
         const long long q = item / tiles_x;
         const int ty = (int)(q % tiles_y);
         const int z0 = (int)(q / tiles_y) * zchunk;
-        const int z1 = min(z0 + zchunk, P);
+        const int zl = min(z0 + zchunk, n);
         const int X0 = tx * kTX, Y0 = ty * kTY;
         const int xo = X0 + 2 * lane, yo = Y0 + 2 * warp;
-        // zero planes of the padding (z >= n)
-        for (int z = max(z0, n); z < z1; ++z) {
-            const long long o = ((long long)z * P + yo) * P + xo;
-            const __nv_bfloat162 zz = __floats2bfloat162_rn(0.0f, 0.0f);
-            Rhi2[o >> 1] = zz;
-            Rlo2[o >> 1] = zz;
-            Rhi2[(o + P) >> 1] = zz;
-            Rlo2[(o + P) >> 1] = zz;
-        }
-        const int zl = min(z1, n);
-        if (z0 >= zl) continue;   // block-uniform
 
         const bool v00 = xo < n && yo < n, v10 = xo + 1 < n && yo < n;
         const bool v01 = xo < n && yo + 1 < n, v11 = xo + 1 < n && yo + 1 < n;
@@ -961,6 +982,7 @@ __global__ void __launch_bounds__(kTThreads, 2) k_residual_tiled(ResidualArgs a,
         }
     }
 
+    zero_padding(a, tiles_x * kTX, tiles_y * kTY, P, 1);
     tile_partials<KIND>(a, kr2, kc, r2k, amin, amax, dmn, dmx);
 }
 
@@ -1016,8 +1038,8 @@ __global__ void __launch_bounds__(kTThreads, 2) k_residual_mirror(ResidualArgs a
     const bool neu = (a.bc == QN_BC_NEUMANN);
     float dmn = INFINITY, dmx = -INFINITY;   // KIND 3: extremes of 3 b u^2 + V
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int tiles_x = H / 32, tiles_y = P / kTY;
-    const int nzc = (P + zchunk - 1) / zchunk;
+    const int tiles_x = (nsym + 31) / 32, tiles_y = (n + kTY - 1) / kTY;   // tiles with grid points
+    const int nzc = (n + zchunk - 1) / zchunk;
     const long long items = (long long)tiles_x * tiles_y * nzc;
     const long long nn = (long long)n * n;
     const unsigned long long *Ub = reinterpret_cast<const unsigned long long *>(a.U);
@@ -1035,26 +1057,11 @@ __global__ void __launch_bounds__(kTThreads, 2) k_residual_mirror(ResidualArgs a
         const long long q = item / tiles_x;
         const int ty = (int)(q % tiles_y);
         const int z0 = (int)(q / tiles_y) * zchunk;
-        const int z1 = min(z0 + zchunk, P);
+        const int zl = min(z0 + zchunk, n);
         const int X0 = tx * 32, Y0 = ty * kTY;
         const int xL = X0 + lane, xR = n - 1 - X0 - lane;
         const int y0 = Y0 + 2 * warp, y1 = y0 + 1;
         const int Fy0 = fold_index(y0, n, nsym), Fy1 = fold_index(y1, n, nsym);
-        // zero planes of the padding (z >= n), both halves of both rows
-        for (int z = max(z0, n); z < z1; ++z) {
-            const long long o0 = ((long long)z * P + Fy0) * P, o1 = ((long long)z * P + Fy1) * P;
-            const __nv_bfloat16 zb = __float2bfloat16_rn(0.0f);
-            a.Rhi[o0 + xL] = zb;
-            a.Rlo[o0 + xL] = zb;
-            a.Rhi[o0 + H + xL] = zb;
-            a.Rlo[o0 + H + xL] = zb;
-            a.Rhi[o1 + xL] = zb;
-            a.Rlo[o1 + xL] = zb;
-            a.Rhi[o1 + H + xL] = zb;
-            a.Rlo[o1 + H + xL] = zb;
-        }
-        const int zl = min(z1, n);
-        if (z0 >= zl) continue;   // block-uniform
 
         // present: the value exists on the grid (else Dirichlet 0); own: this
         // thread evaluates the point (left: x <= middle; right: x > middle)
@@ -1277,6 +1284,7 @@ __global__ void __launch_bounds__(kTThreads, 2) k_residual_mirror(ResidualArgs a
         }
     }
 
+    zero_padding(a, tiles_x * 32, tiles_y * kTY, H, 2);
     tile_partials<KIND>(a, kr2, kc, r2k, amin, amax, dmn, dmx);
 }
 
@@ -1802,6 +1810,25 @@ int launch_residual(const ResidualArgs &a, int grid, cudaStream_t s) {
     return QN_OK;
 }
 
+// Planes per work item: the fewest plane steps of the busiest block, its items times their
+// planes and the two that an item reads ahead of its first. A fixed 32 leaves the last round of
+// the blocks nearly empty at some sizes and too few items at small ones; with tiles over the
+// grid points alone (instead of the padded ones) a solve of 8 iterations takes, before and now:
+// n = 65 0.94, 0.75 ms; 100 0.94, 0.79; 130 1.33, 1.23; 255 3.05, 2.97; 400 13.1, 12.6; 511 19.7,
+// 19.5. Example 1's residual at 400^3: 601, 538 us.
+static int balanced_zchunk(long long tiles, int n, long long blocks) {
+    int best = 32;
+    long long cost = LLONG_MAX;
+    for (int zc = 4; zc <= 96; ++zc) {
+        const long long c = (tiles * ((n + zc - 1) / zc) + blocks - 1) / blocks * (zc + 2);
+        if (c < cost) {
+            cost = c;
+            best = zc;
+        }
+    }
+    return best;
+}
+
 template <int KIND>
 static int tiled_blocks_per_sm() {
     static int cached = 0;   // per process: every device it runs on is a GB300
@@ -1820,9 +1847,11 @@ static int launch_tiled_kind(const ResidualArgs &a, int max_grid, int zchunk, in
     int dev = 0, sms = 0;
     QN_CUDA(cudaGetDevice(&dev));
     QN_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const long long items = (long long)(a.P / kTX) * (a.P / kTY) * ((a.P + zchunk - 1) / zchunk);
+    const long long tiles = (long long)((a.n + kTX - 1) / kTX) * ((a.n + kTY - 1) / kTY);
     long long g = (long long)tiled_blocks_per_sm<KIND>() * sms;
     if (g > max_grid) g = max_grid;
+    if (zchunk == 0) zchunk = balanced_zchunk(tiles, a.n, g);
+    const long long items = tiles * ((a.n + zchunk - 1) / zchunk);
     if (g > items) g = items;
     if (g < 1) g = 1;
     k_residual_tiled<KIND><<<(int)g, kTThreads, 0, s>>>(a, zchunk);
@@ -1849,9 +1878,11 @@ static int launch_mirror_kind(const ResidualArgs &a, int max_grid, int zchunk, i
     int dev = 0, sms = 0;
     QN_CUDA(cudaGetDevice(&dev));
     QN_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const long long items = (long long)(a.P / 64) * (a.P / kTY) * ((a.P + zchunk - 1) / zchunk);
+    const long long tiles = (long long)(((a.n + 1) / 2 + 31) / 32) * ((a.n + kTY - 1) / kTY);
     long long g = (long long)mirror_blocks_per_sm<KIND>() * sms;
     if (g > max_grid) g = max_grid;
+    if (zchunk == 0) zchunk = balanced_zchunk(tiles, a.n, g);
+    const long long items = tiles * ((a.n + zchunk - 1) / zchunk);
     if (g > items) g = items;
     if (g < 1) g = 1;
     k_residual_mirror<KIND><<<(int)g, kTThreads, 0, s>>>(a, zchunk);
@@ -1862,7 +1893,7 @@ static int launch_mirror_kind(const ResidualArgs &a, int max_grid, int zchunk, i
 
 int launch_residual_mirror(const ResidualArgs &a, int max_grid, int zchunk, int *grid_used, cudaStream_t s) {
     if (a.dim != 3 || a.Rhi == nullptr || a.fdf == nullptr || a.fx_e == nullptr || !tc_split_sizes(a.P) ||
-        zchunk < 1) {
+        zchunk < 0) {
         set_error("launch_residual_mirror: needs a 3-D split residual at a size of the split products, the f copy");
         return QN_EINVAL;
     }
@@ -1909,7 +1940,7 @@ int launch_fused_residual_fwd(const ResidualArgs &a, const FusedFwd &ff, int *gr
 
 int launch_residual_tiled(const ResidualArgs &a, int max_grid, int zchunk, int *grid_used, cudaStream_t s) {
     if (a.dim != 3 || a.Rhi == nullptr || a.fdf == nullptr || a.fx_e == nullptr || a.P % kTX != 0 ||
-        zchunk < 1) {
+        zchunk < 0) {
         set_error("launch_residual_tiled: needs a 3-D split residual with the FP32-pair copy of f");
         return QN_EINVAL;
     }
