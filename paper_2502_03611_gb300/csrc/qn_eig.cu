@@ -212,16 +212,49 @@ __global__ void __launch_bounds__(256) k_eig_pass1(const double *__restrict__ U,
 
 // s = 1/||U~|| and lambda_n of U = s U~; the scale |lambda_n| of the stop test.
 __global__ void __launch_bounds__(256) k_eig_finalize1(const double *partials, int nparts, double hd, DevState *st) {
-    if (state_done(st)) return;
-    Sum4 acc{0.0, 0.0, 0.0, 0.0};
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
-        acc.a += partials[4 * i + 0];
-        acc.b += partials[4 * i + 1];
-        acc.mn += partials[4 * i + 2];
+    // the first three records of every thread are read together with the state
+    constexpr int kAhead = 3;
+    const double2 *rec = reinterpret_cast<const double2 *>(partials);
+    double2 v[kAhead];
+    double q[kAhead];
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) {
+        const int i = threadIdx.x + 256 * k;
+        if (i < nparts) {
+            v[k] = rec[2 * i];
+            q[k] = partials[4 * i + 2];
+        }
     }
-    acc = block_sum3(acc);
+    if (state_done(st)) return;
+    __shared__ double sums[3][256], tot[3];
+    double e1 = 0.0, e4 = 0.0, uu = 0.0;
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k)
+        if (threadIdx.x + 256 * k < nparts) {
+            e1 = (k == 0) ? v[k].x : e1 + v[k].x;
+            e4 = (k == 0) ? v[k].y : e4 + v[k].y;
+            uu = (k == 0) ? q[k] : uu + q[k];
+        }
+    for (int i = threadIdx.x + 256 * kAhead; i < nparts; i += 256) {
+        e1 += partials[4 * i + 0];
+        e4 += partials[4 * i + 1];
+        uu += partials[4 * i + 2];
+    }
+    sums[0][threadIdx.x] = e1;
+    sums[1][threadIdx.x] = e4;
+    sums[2][threadIdx.x] = uu;
+    __syncthreads();
+    const int warp = threadIdx.x >> 5;
+    if (warp < 3) {   // one sum per warp, eight values per lane (FP64 takes its pipe 16 cycles per warp)
+        const double *p = sums[warp] + (threadIdx.x & 31);
+        double t = ((p[0] + p[128]) + (p[32] + p[160])) + ((p[64] + p[192]) + (p[96] + p[224]));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if ((threadIdx.x & 31) == 0) tot[warp] = t;
+    }
+    __syncthreads();
     if (threadIdx.x != 0) return;
-    const double E1 = acc.a, E4 = acc.b, Q = acc.mn;
+    const double E1 = tot[0], E4 = tot[1], Q = tot[2];
     const double s2 = 1.0 / (hd * Q);                  // ||s U~||^2 = s^2 h^d Q = 1
     const double sc = sqrt(s2);
     st->eig_scale = sc;

@@ -63,6 +63,37 @@ __device__ Red4 block_reduce(Red4 v) {
     return v;
 }
 
+// Sum of 256 values in shared memory by one warp: eight per lane, then the warp. An FP64
+// instruction takes its pipe 16 cycles per warp, so a tree over all eight warps (41 + 5 adds)
+// costs three times these 12.
+__device__ __forceinline__ double warp_sum_256(const double *v) {
+    const int l = threadIdx.x & 31;
+    double t[4];
+#pragma unroll
+    for (int w = 0; w < 4; ++w) t[w] = v[l + 32 * w] + v[l + 32 * (w + 4)];
+    double r = (t[0] + t[1]) + (t[2] + t[3]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    return r;
+}
+
+// Doubles as integers of the same order; a NaN is passed over (`none`).
+__device__ __forceinline__ unsigned long long order_key(double v, unsigned long long none) {
+    const long long b = __double_as_longlong(v);
+    if ((b & 0x7FFFFFFFFFFFFFFFll) > 0x7FF0000000000000ll) return none;
+    return (unsigned long long)(b ^ ((b >> 63) | (1ll << 63)));
+}
+__device__ __forceinline__ double key_value(unsigned long long k) {
+    return __longlong_as_double((long long)((k >> 63) ? k ^ (1ull << 63) : ~k));
+}
+
+__device__ __forceinline__ unsigned long long redux_max_u64(unsigned long long v) {
+    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(v >> 32));
+    const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(v >> 32) == hi ? (unsigned)v : 0u);
+    return (unsigned long long)hi << 32 | lo;
+}
+__device__ __forceinline__ unsigned long long redux_min_u64(unsigned long long v) { return ~redux_max_u64(~v); }
+
 __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -270,77 +301,83 @@ __global__ void __launch_bounds__(256) k_prep_split(const double *__restrict__ U
     unsigned long long umax = 0ull;
     float s2h = 0.0f, s2l = 0.0f;   // sum f^2 as a float pair (MIRROR)
     if (MIRROR) {
-        // four rows per step, their loads issued together (the pass is
-        // latency-bound with one row per step); rows < P^2 <= 2^22: 32-bit index math
-        constexpr int kRows = 4;
+        // four mirror pairs per thread and step, their loads issued together (the pass is
+        // latency-bound with one), and all threads busy whatever P / 2 is: a thread per position
+        // of a row left half the block idle at P = 256 (255^3: 175 us, now 99; 511^3: 789, now 737)
+        constexpr unsigned kRows = 4, kStep = 256 * kRows;
         float4 *f4 = reinterpret_cast<float4 *>(fdf);
-        const unsigned int urows = (unsigned int)rows, uP = (unsigned int)P;
-        for (unsigned int row0 = blockIdx.x; row0 < urows; row0 += (unsigned int)kRows * gridDim.x) {
-            int ys[kRows], zs[kRows];
-#pragma unroll
-            for (int g = 0; g < kRows; ++g) {
-                const unsigned int row = row0 + (unsigned int)g * gridDim.x;
-                zs[g] = (int)(row / uP);
-                ys[g] = (int)(row - (unsigned int)zs[g] * uP);
+        const unsigned uP = (unsigned)P, uH = (unsigned)H;
+        const size_t total = (size_t)rows * uH, stride = (size_t)gridDim.x * kStep;
+        const unsigned long long srow = stride / uH;
+        const unsigned soff = (unsigned)(stride - srow * uH);
+        size_t base = (size_t)blockIdx.x * kStep;
+        unsigned long long brow = base / uH;
+        unsigned boff = (unsigned)(base - brow * uH);   // base = brow * H + boff
+        for (; base < total; base += stride, brow += srow, boff += soff) {
+            if (boff >= uH) {
+                boff -= uH;
+                ++brow;
             }
-            for (int i = threadIdx.x; i < H; i += blockDim.x) {
-                double fa[kRows], fb[kRows], ua[kRows], ub[kRows];
-                bool oka[kRows], okb[kRows];
+            int ys[kRows], zs[kRows], is[kRows];
+            double fa[kRows], fb[kRows], ua[kRows], ub[kRows];
+            bool oka[kRows], okb[kRows];
 #pragma unroll
-                for (int g = 0; g < kRows; ++g) {
-                    const unsigned int row = row0 + (unsigned int)g * gridDim.x;
-                    const int y = ys[g], z = zs[g];
-                    const bool row_ok = row < urows && (y < n) && (z < n);
-                    const long long cbase = ((long long)z * n + y) * n;
-                    oka[g] = row_ok && i < nsym;
-                    okb[g] = row_ok && i < nanti;
-                    fa[g] = oka[g] ? __ldg(f + cbase + i) : 0.0;
-                    ua[g] = oka[g] ? __ldg(U + cbase + i) : 0.0;
-                    fb[g] = okb[g] ? __ldg(f + cbase + (n - 1 - i)) : 0.0;
-                    ub[g] = okb[g] ? __ldg(U + cbase + (n - 1 - i)) : 0.0;
+            for (unsigned g = 0; g < kRows; ++g) {
+                const unsigned o = boff + threadIdx.x + g * 256u, dr = o / uH;
+                const unsigned row = (unsigned)brow + dr;   // < P^2 + 2 H + 1024
+                const int i = (int)(o - dr * uH), z = (int)(row / uP), y = (int)(row - (unsigned)z * uP);
+                const bool row_ok = (y < n) && (z < n);
+                const long long cbase = ((long long)z * n + y) * n;
+                is[g] = i;
+                zs[g] = z;
+                ys[g] = y;
+                oka[g] = row_ok && i < nsym;
+                okb[g] = row_ok && i < nanti;
+                fa[g] = oka[g] ? __ldg(f + cbase + i) : 0.0;
+                ua[g] = oka[g] ? __ldg(U + cbase + i) : 0.0;
+                fb[g] = okb[g] ? __ldg(f + cbase + (n - 1 - i)) : 0.0;
+                ub[g] = okb[g] ? __ldg(U + cbase + (n - 1 - i)) : 0.0;
+            }
+#pragma unroll
+            for (unsigned g = 0; g < kRows; ++g) {
+                if (base + threadIdx.x + g * 256u >= total) break;
+                float2 a = make_float2(0.0f, 0.0f), b = a;
+                if (oka[g]) {
+                    a = f_pair(fa[g], &st->fx_fbad);
+                    const unsigned long long ab = abs_bits(ua[g]);
+                    umax = ab > umax ? ab : umax;
                 }
-#pragma unroll
-                for (int g = 0; g < kRows; ++g) {
-                    const unsigned int row = row0 + (unsigned int)g * gridDim.x;
-                    if (row >= urows) break;
-                    float2 a = make_float2(0.0f, 0.0f), b = a;
-                    if (oka[g]) {
-                        a = f_pair(fa[g], &st->fx_fbad);
-                        const unsigned long long ab = abs_bits(ua[g]);
-                        umax = ab > umax ? ab : umax;
-                    }
-                    if (okb[g]) {
-                        b = f_pair(fb[g], &st->fx_fbad);
-                        const unsigned long long ab = abs_bits(ub[g]);
-                        umax = ab > umax ? ab : umax;
-                    }
-                    // f^2 = hi^2 + 2 hi lo (+ lo^2, below 2^-46 of it) as a float pair
-                    {
-                        float p = __fmul_rn(a.x, a.x), e = __fmaf_rn(a.x, a.x, -p);
-                        e = __fmaf_rn(__fadd_rn(a.x, a.x), a.y, e);
-                        const float q = __fmul_rn(b.x, b.x);
-                        float eq = __fmaf_rn(b.x, b.x, -q);
-                        eq = __fmaf_rn(__fadd_rn(b.x, b.x), b.y, eq);
-                        float t, te;
-                        two_sum(p, q, t, te);
-                        float s, se;
-                        two_sum(s2h, t, s, se);
-                        s2l = __fadd_rn(s2l, __fadd_rn(se, __fadd_rn(te, __fadd_rn(e, eq))));
-                        s2h = s;
-                    }
-                    f4[(long long)row * H + i] = make_float4(a.x, a.y, b.x, b.y);
-                    if (Rhi != nullptr) {
-                        // split order along x, folded rows (rows of the padding stay in place)
-                        const int y = ys[g], z = zs[g];
-                        const int Fy = (y >= n) ? y : (y < nsym ? 2 * y : 2 * (n - 1 - y) + 1);
-                        const int Fz = (z >= n) ? z : (z < nsym ? 2 * z : 2 * (n - 1 - z) + 1);
-                        const long long o = ((long long)Fz * P + Fy) * P;
-                        // (+ 0.0f: a zero f gives +0, as the residual's arithmetic does)
-                        const float ra = oka[g] ? __fadd_rn(-a.x, 0.0f) : 0.0f;
-                        const float rb = okb[g] ? __fadd_rn(-b.x, 0.0f) : 0.0f;
-                        split_bf16(__fadd_rn(ra, rb), Rhi[o + i], Rlo[o + i]);
-                        split_bf16(okb[g] ? __fsub_rn(ra, rb) : 0.0f, Rhi[o + H + i], Rlo[o + H + i]);
-                    }
+                if (okb[g]) {
+                    b = f_pair(fb[g], &st->fx_fbad);
+                    const unsigned long long ab = abs_bits(ub[g]);
+                    umax = ab > umax ? ab : umax;
+                }
+                // f^2 = hi^2 + 2 hi lo (+ lo^2, below 2^-46 of it) as a float pair
+                {
+                    float p = __fmul_rn(a.x, a.x), e = __fmaf_rn(a.x, a.x, -p);
+                    e = __fmaf_rn(__fadd_rn(a.x, a.x), a.y, e);
+                    const float q = __fmul_rn(b.x, b.x);
+                    float eq = __fmaf_rn(b.x, b.x, -q);
+                    eq = __fmaf_rn(__fadd_rn(b.x, b.x), b.y, eq);
+                    float t, te;
+                    two_sum(p, q, t, te);
+                    float s, se;
+                    two_sum(s2h, t, s, se);
+                    s2l = __fadd_rn(s2l, __fadd_rn(se, __fadd_rn(te, __fadd_rn(e, eq))));
+                    s2h = s;
+                }
+                f4[base + threadIdx.x + g * 256u] = make_float4(a.x, a.y, b.x, b.y);
+                if (Rhi != nullptr) {
+                    // split order along x, folded rows (rows of the padding stay in place)
+                    const int y = ys[g], z = zs[g], i = is[g];
+                    const int Fy = (y >= n) ? y : (y < nsym ? 2 * y : 2 * (n - 1 - y) + 1);
+                    const int Fz = (z >= n) ? z : (z < nsym ? 2 * z : 2 * (n - 1 - z) + 1);
+                    const long long o = ((long long)Fz * P + Fy) * P;
+                    // (+ 0.0f: a zero f gives +0, as the residual's arithmetic does)
+                    const float ra = oka[g] ? __fadd_rn(-a.x, 0.0f) : 0.0f;
+                    const float rb = okb[g] ? __fadd_rn(-b.x, 0.0f) : 0.0f;
+                    split_bf16(__fadd_rn(ra, rb), Rhi[o + i], Rlo[o + i]);
+                    split_bf16(okb[g] ? __fsub_rn(ra, rb) : 0.0f, Rhi[o + H + i], Rlo[o + H + i]);
                 }
             }
         }
@@ -367,10 +404,13 @@ __global__ void __launch_bounds__(256) k_prep_split(const double *__restrict__ U
         }
     }
     const unsigned long long bm = block_max_u64(umax);
-    Red4 acc{0.0, f2, 0.0, 0.0};
-    acc = block_reduce(acc);
+    __shared__ double sum[256];
+    sum[threadIdx.x] = f2;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    f2 = warp_sum_256(sum);
     if (threadIdx.x == 0) {
-        partials[4ll * blockIdx.x + 1] = acc.f2;
+        partials[4ll * blockIdx.x + 1] = f2;
         atomicMax(&st->umax_scan, bm);
     }
 }
@@ -378,11 +418,15 @@ __global__ void __launch_bounds__(256) k_prep_split(const double *__restrict__ U
 // ||f|| (fixed-order sum of the partials), the scale of the FP32 norm sums
 // and the fixed-point exponent for the first residual.
 __global__ void __launch_bounds__(256) k_prep_split_finish(const double *partials, int nparts, DevState *st) {
-    Red4 acc{0.0, 0.0, 0.0, 0.0};
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) acc.f2 += partials[4 * i + 1];
-    acc = block_reduce(acc);
+    __shared__ double sum[256];
+    double f2 = 0.0;
+    for (int i = threadIdx.x; i < nparts; i += 256) f2 += partials[4 * i + 1];
+    sum[threadIdx.x] = f2;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    f2 = warp_sum_256(sum);
     if (threadIdx.x != 0) return;
-    const double fn = sqrt(acc.f2);
+    const double fn = sqrt(f2);
     st->f_norm = fn;
     const double rms = (st->npts > 0.0) ? fn / sqrt(st->npts) : 0.0;
     const int k = (rms > 0.0 && rms < INFINITY) ? ilogb(rms) : 0;
@@ -440,27 +484,71 @@ __global__ void k_umax_finish(DevState *st) {
     st->umax_scan = 0ull;
 }
 
+// One block, a chain of latencies: the state and the first three records of every thread are
+// read together, the sums are taken by one warp each (warp_sum_256) and the extremes as integers
+// (8.5 us under a profiler with a tree over all warps and serial state reads, 5.6 so).
 __global__ void __launch_bounds__(256) k_finalize(const double *partials, int nparts, DevState *st,
                                                   qn_stats *hist, int hist_cap, double b,
                                                   double lam, int update_state, int use_saved_fnorm,
                                                   int mode) {
     const bool pot = (mode == 1), eig = (mode == 2);
-    if (update_state && *(volatile int *)&st->done) return;
-    Red4 acc{0.0, 0.0, INFINITY, 0.0};
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
-        acc.r2 += partials[4 * i + 0];
-        acc.f2 += partials[4 * i + 1];
-        acc.mn = fmin(acc.mn, partials[4 * i + 2]);
-        acc.mx = fmax(acc.mx, partials[4 * i + 3]);
+    constexpr int kAhead = 3;
+    const double2 *rec = reinterpret_cast<const double2 *>(partials);
+    double2 v[kAhead][2];
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) {
+        const int i = threadIdx.x + 256 * k;
+        if (i < nparts) {
+            v[k][0] = rec[2 * i];
+            v[k][1] = rec[2 * i + 1];
+        }
     }
-    acc = block_reduce(acc);
+    DevState d = *st;
+    if (update_state && d.done) return;
+    __shared__ double sums[2][256], root[3];
+    __shared__ unsigned long long ext[2][8];
+    const unsigned long long none_min = order_key(INFINITY, 0ull), none_max = order_key(0.0, 0ull);
+    double r2 = 0.0, f2 = 0.0;
+    unsigned long long kmin = none_min, kmax = none_max;
+    auto add = [&](double2 x, double2 y, bool first) {
+        r2 = first ? x.x : r2 + x.x;
+        if (!use_saved_fnorm) f2 += x.y;
+        kmin = min(kmin, order_key(y.x, none_min));
+        kmax = max(kmax, order_key(y.y, none_max));
+    };
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k)
+        if (threadIdx.x + 256 * k < nparts) add(v[k][0], v[k][1], k == 0);
+    for (int i = threadIdx.x + 256 * kAhead; i < nparts; i += 256) add(rec[2 * i], rec[2 * i + 1], false);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    sums[0][threadIdx.x] = r2;
+    sums[1][threadIdx.x] = f2;
+    kmin = redux_min_u64(kmin);
+    kmax = redux_max_u64(kmax);
+    if (lane == 0) {
+        ext[0][warp] = kmin;
+        ext[1][warp] = kmax;
+    }
+    __syncthreads();
+    // ||r|| and, in warps beside it, ||f|| and sqrt(max)
+    Red4 acc;
+    kmin = redux_min_u64(ext[0][lane & 7]);
+    kmax = redux_max_u64(ext[1][lane & 7]);
+    acc.mn = key_value(kmin);
+    acc.mx = key_value(kmax);
+    if (warp < 3) {
+        const double arg = (warp == 2) ? acc.mx : (warp == 1 && use_saved_fnorm) ? 0.0 : warp_sum_256(sums[warp]);
+        const double q = sqrt(arg);
+        if (lane == 0) root[warp] = q;
+    }
+    __syncthreads();
+    const double res = root[0], fn = use_saved_fnorm ? d.f_norm : root[1], umax = root[2];
     if (threadIdx.x != 0) return;
-    const double res = sqrt(acc.r2);
-    const double fn = use_saved_fnorm ? st->f_norm : sqrt(acc.f2);
+    d.f_norm = fn;
     if (update_state && !use_saved_fnorm) {
         st->f_norm = fn;
         // scale of the FP32 sum of r^2 in the later iterations: 2^k ~ RMS(f)
-        const double rms = (st->npts > 0.0) ? fn / sqrt(st->npts) : 0.0;
+        const double rms = (d.npts > 0.0) ? fn / sqrt(d.npts) : 0.0;
         int k = (rms > 0.0 && rms < INFINITY) ? ilogb(rms) : 0;
         st->r2_exp = k < -120 ? -120 : (k > 120 ? 120 : k);
     }
@@ -468,14 +556,14 @@ __global__ void __launch_bounds__(256) k_finalize(const double *partials, int np
     const double fa = (pot || eig) ? acc.mn : 3.0 * b * acc.mn, fb = (pot || eig) ? acc.mx : 3.0 * b * acc.mx;
     const double fu_min = fmin(fa, fb), fu_max = fmax(fa, fb);
     // eigen solves: (N_h)_U = diag(lam + 3 b U^2 + V) - lambda_n (extremes from pass 2)
-    const double beta = (st->beta_mode == QN_BETA_FIXED) ? st->beta_value
-                                                         : 0.5 * (fu_min + fu_max) - (eig ? st->eig_lambda : 0.0);
+    const double beta = (d.beta_mode == QN_BETA_FIXED) ? d.beta_value
+                                                       : 0.5 * (fu_min + fu_max) - (eig ? d.eig_lambda : 0.0);
     double rel;
     if (fn > 0.0)
         rel = res / fn;
     else
         rel = (res == 0.0) ? 0.0 : INFINITY;
-    const int it = st->it;
+    const int it = d.it;
     if (hist != nullptr && it >= 0 && it < hist_cap) {
         qn_stats s;
         s.res_norm = res;
@@ -484,7 +572,7 @@ __global__ void __launch_bounds__(256) k_finalize(const double *partials, int np
         s.fu_max = fu_max;
         s.beta = beta;
         s.rel = rel;
-        s.lambda = eig ? st->eig_lambda : 0.0;
+        s.lambda = eig ? d.eig_lambda : 0.0;
         hist[it] = s;
     }
     if (!update_state) return;
@@ -492,20 +580,20 @@ __global__ void __launch_bounds__(256) k_finalize(const double *partials, int np
     // of this iterate (sqrt of max U^2 has at least max|U|'s exponent: the
     // rounding of u^2 can only carry it up)
     if (pot || eig) {   // max|U| gathered by the residual passes (atomicMax of bit patterns)
-        st->fx_e = fx_exponent(st->umax_scan, st);
+        st->fx_e = fx_exponent(d.umax_scan, &d);
         st->umax_scan = 0ull;
     } else {
-        st->fx_e = (acc.mx < INFINITY) ? fx_exponent((unsigned long long)__double_as_longlong(sqrt(acc.mx)), st) : 0;
+        st->fx_e = (acc.mx < INFINITY) ? fx_exponent((unsigned long long)__double_as_longlong(umax), &d) : 0;
     }
     st->beta = beta;
     st->shift = eig ? beta : lam + beta;   // eigen solves: lam is part of f, not of A_h
-    if (rel <= st->tol) {
+    if (rel <= d.tol) {
         st->status = QN_OK;
         st->done = 1;
     } else if (!isfinite(rel) || rel > 1e8 || !isfinite(beta)) {
         st->status = QN_EDIVERGED;
         st->done = 1;
-    } else if (it >= st->max_it) {
+    } else if (it >= d.max_it) {
         st->status = QN_ENOTCONV;
         st->done = 1;
     } else {
@@ -673,16 +761,58 @@ template <int KIND>
 __device__ __forceinline__ void tile_partials(const ResidualArgs &a, float kr2, float kc, int r2k,
                                               unsigned long long amin, unsigned long long amax, float dmn,
                                               float dmx) {
+    // FP64 work by one warp (warp_sum_256) and one thread; the extremes as integers and FP32
+    __shared__ double sum[256];
+    __shared__ unsigned long long ext[2][8];
+    __shared__ float dext[2][8];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    sum[threadIdx.x] = f2d_exact(kr2) - f2d_exact(kc);
+    amin = redux_min_u64(amin);
+    amax = redux_max_u64(amax);
+    if (KIND == 3) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            dmn = fminf(dmn, __shfl_xor_sync(0xffffffffu, dmn, o));
+            dmx = fmaxf(dmx, __shfl_xor_sync(0xffffffffu, dmx, o));
+        }
+    }
+    if (lane == 0) {
+        ext[0][warp] = amin;
+        ext[1][warp] = amax;
+        dext[0][warp] = dmn;
+        dext[1][warp] = dmx;
+    }
+    __syncthreads();
+    if (warp != 0) return;
+    const double r2 = warp_sum_256(sum);
+    amin = redux_min_u64(ext[0][lane & 7]);
+    amax = redux_max_u64(ext[1][lane & 7]);
+    if (lane != 0) return;
+    double *p = a.partials + 4ll * blockIdx.x;
+    p[0] = ldexp(r2, 2 * r2k);
+    p[1] = 0.0;
+    if (KIND == 3) {
+        for (int w = 1; w < 8; ++w) {
+            dmn = fminf(dmn, dext[0][w]);
+            dmx = fmaxf(dmx, dext[1][w]);
+        }
+        p[2] = (double)dmn;
+        p[3] = fmax(0.0, (double)dmx);
+        atomicMax(a.umax_scan, amax);
+    } else {
+        const double umin = __longlong_as_double((long long)amin), umax = __longlong_as_double((long long)amax);
+        p[2] = (amin == 0x7FFFFFFFFFFFFFFFull) ? INFINITY : umin * umin;
+        p[3] = umax * umax;
+    }
+}
+
+// The partial record of a block of any size (k_fused_res_fwd).
+__device__ __forceinline__ void block_partials(const ResidualArgs &a, float kr2, float kc, int r2k,
+                                               unsigned long long amin, unsigned long long amax) {
     const double umin = __longlong_as_double((long long)amin);
     const double umax = __longlong_as_double((long long)amax);
     Red4 acc{ldexp((double)kr2 - (double)kc, 2 * r2k), 0.0,
              (amin == 0x7FFFFFFFFFFFFFFFull) ? INFINITY : umin * umin, umax * umax};
-    if (KIND == 3) {
-        acc.mn = (double)dmn;
-        acc.mx = (double)dmx;
-        const unsigned long long bm = block_max_u64(amax);
-        if (threadIdx.x == 0) atomicMax(a.umax_scan, bm);
-    }
     acc = block_reduce(acc);
     if (threadIdx.x == 0) {
         double *p = a.partials + 4ll * blockIdx.x;
@@ -1720,7 +1850,7 @@ __global__ void __maxnreg__(96) k_fused_res_fwd(ResidualArgs a, FusedFwd ff) {
         }
     }
 
-    tile_partials<KIND>(a, kr2, kc, r2k, amin, amax, INFINITY, -INFINITY);
+    block_partials(a, kr2, kc, r2k, amin, amax);
     ptx::tc_fence_before();
     __syncthreads();
     if (warp == 1) {
