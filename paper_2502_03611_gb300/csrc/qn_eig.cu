@@ -23,7 +23,10 @@
 // self-adjoint in it, so F is orthogonal to U. All reductions are per-block
 // partials summed in a fixed order (deterministic: graph replay is bitwise
 // the same as plain launches).
+#include <limits.h>
 #include <math.h>
+
+#include <algorithm>
 
 #include "qn_df.cuh"
 #include "qn_internal.h"
@@ -500,15 +503,16 @@ __global__ void __launch_bounds__(256) k_eig_pass1_df(const double *__restrict__
 
 // ---- tiled pass 1 (3-D, float pairs) ------------------------------------------------------
 // The arithmetic of k_eig_pass1_df with each value converted to fixed point once: a block
-// owns a 32 x 8 (x, y) tile of a run of z planes, one warp per y row, and walks z. The
+// owns a W x H (x, y) tile of a run of z planes, a thread per column of it, and walks z. The
 // tile's plane z and its x / y halo sit in shared memory (double-buffered), the z - 1 and
 // z + 1 values of the thread's own column in registers; the next plane's loads are in
 // flight while the current one is evaluated. A node takes the FP64 path when a value of
 // plane z (anywhere in the tile: one block-wide flag) or of its own column at z - 1, z + 1
-// lies beyond the fixed-point exponent.
-constexpr int kP1W = 32, kP1H = 8;
-constexpr int kP1SW = kP1W + 2, kP1SH = kP1H + 2;
-constexpr int kP1Halo = 2 * kP1W + 2 * kP1H;   // 80 halo values per plane (no corners)
+// lies beyond the fixed-point exponent. The kernel is bound by instruction issue (about 230 a
+// node), so W and H (W H <= 256) are the ones that cover the grid with the fewest tiles
+// (pass1_tile): at n = 100, 25 x 10 leaves 2 % of the threads idle where 32 x 8 left 25 %
+// (23.9 us, now 18.5, the planes per item chosen by balanced_zchunk).
+constexpr int kP1Cells = 66 * 6;   // most (W + 2)(H + 2) of the tiles: 64 x 4
 
 __device__ __forceinline__ int ghost_of(int i, int n, bool neu) {
     return neu ? (i == -1 ? 1 : (i == n ? n - 2 : i)) : i;
@@ -527,38 +531,41 @@ __device__ __forceinline__ unsigned long long ld_node3(const unsigned long long 
 
 template <bool NEU>
 __global__ void __launch_bounds__(256, 3) k_eig_pass1_tiled(const double *__restrict__ U, float2 *__restrict__ lin,
-                                                            int n, int zchunk, double inv_h2, double lam,
+                                                            int n, int W, int H, int zchunk, double inv_h2, double lam,
                                                             float2 lam2, double b, const double *__restrict__ pot,
                                                             const double *__restrict__ vrow,
                                                             const float2 *__restrict__ pot2,
                                                             const float2 *__restrict__ vrow2,
                                                             double *__restrict__ partials, const DevState *st) {
     if (state_done(st)) return;
-    __shared__ long long sp[2][kP1SH][kP1SW];
+    __shared__ long long sp[2][kP1Cells];
     const int E = st->fx_e;
     const float scale = __int_as_float(E != 0 ? ((E - 1075 - kFxG + 127) << 23) : 0);
     const float ih = __double2float_rn(inv_h2), il = __double2float_rn(inv_h2 - (double)ih);
     const float2 ih2 = make_float2(ih, il);
     const unsigned long long *Ub = reinterpret_cast<const unsigned long long *>(U);
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int t = threadIdx.x, ly = t / W, lx = t - ly * W, pitch = W + 2;
+    const bool active = ly < H;
+    const int own_at = active ? (ly + 1) * pitch + lx + 1 : pitch + 1;   // this thread's shared slot
     // this thread's halo slot: the rows above / below the tile, then the columns left / right
-    const bool halo = t < kP1Halo;
+    const bool halo = t < 2 * (W + H);
     int hr, hc;
-    if (t < kP1W) {
+    if (t < W) {
         hr = 0;
         hc = t + 1;
-    } else if (t < 2 * kP1W) {
-        hr = kP1SH - 1;
-        hc = t - kP1W + 1;
-    } else if (t < 2 * kP1W + kP1H) {
-        hr = t - 2 * kP1W + 1;
+    } else if (t < 2 * W) {
+        hr = H + 1;
+        hc = t - W + 1;
+    } else if (t < 2 * W + H) {
+        hr = t - 2 * W + 1;
         hc = 0;
     } else {
-        hr = t - 2 * kP1W - kP1H + 1;
-        hc = kP1SW - 1;
+        hr = t - 2 * W - H + 1;
+        hc = W + 1;
     }
     if (!halo) hr = hc = 0;
-    const int tiles_x = (n + kP1W - 1) / kP1W, tiles_y = (n + kP1H - 1) / kP1H;
+    const int halo_at = hr * pitch + hc;
+    const int tiles_x = (n + W - 1) / W, tiles_y = (n + H - 1) / H;
     const int nzc = (n + zchunk - 1) / zchunk;
     const long long items = (long long)tiles_x * tiles_y * nzc;
     float2 e1 = make_float2(0.f, 0.f), e4 = e1, q = e1;
@@ -568,14 +575,14 @@ __global__ void __launch_bounds__(256, 3) k_eig_pass1_tiled(const double *__rest
         const int ty = (int)(rest % tiles_y);
         const int z0 = (int)(rest / tiles_y) * zchunk;
         const int z1 = min(z0 + zchunk, n);
-        const int x = tx * kP1W + lane, y = ty * kP1H + w;
-        const int hx = tx * kP1W + hc - 1, hy = ty * kP1H + hr - 1;
+        const int x = active ? tx * W + lx : n + 1, y = ty * H + ly;   // (n + 1: reads 0)
+        const int hx = tx * W + hc - 1, hy = ty * H + hr - 1;
         const bool own = x < n && y < n;
         unsigned bm = (E == 0) ? 1u : 0u, bc = bm, bh = bm;   // bad flags: own z-1, own z, plane z (local)
         long long fmv = fx_of(ld_node3<NEU>(Ub, z0 - 1, y, x, n), E, bm);
         long long fc = fx_of(ld_node3<NEU>(Ub, z0, y, x, n), E, bc);
-        sp[0][w + 1][lane + 1] = fc;
-        if (halo) sp[0][hr][hc] = fx_of(ld_node3<NEU>(Ub, z0, hy, hx, n), E, bh);
+        if (active) sp[0][own_at] = fc;
+        if (halo) sp[0][halo_at] = fx_of(ld_node3<NEU>(Ub, z0, hy, hx, n), E, bh);
         bh |= bc;
         unsigned long long nO = ld_node3<NEU>(Ub, z0 + 1, y, x, n);
         unsigned long long nH = halo ? ld_node3<NEU>(Ub, z0 + 1, hy, hx, n) : 0ull;
@@ -585,8 +592,8 @@ __global__ void __launch_bounds__(256, 3) k_eig_pass1_tiled(const double *__rest
             unsigned bp = (E == 0) ? 1u : 0u;
             const long long fp = fx_of(nO, E, bp);
             bh = bp;
-            sp[buf ^ 1][w + 1][lane + 1] = fp;
-            if (halo) sp[buf ^ 1][hr][hc] = fx_of(nH, E, bh);
+            if (active) sp[buf ^ 1][own_at] = fp;
+            if (halo) sp[buf ^ 1][halo_at] = fx_of(nH, E, bh);
             if (z + 1 < z1) {   // prefetch plane z + 2
                 nO = ld_node3<NEU>(Ub, z + 2, y, x, n);
                 if (halo) nH = ld_node3<NEU>(Ub, z + 2, hy, hx, n);
@@ -595,8 +602,8 @@ __global__ void __launch_bounds__(256, 3) k_eig_pass1_tiled(const double *__rest
                 const long long c = ((long long)z * n + y) * n + x;
                 float2 lv, up;
                 if (!(plane_bad || bm || bp)) {
-                    const long long lapfx = 6 * fc - sp[buf][w + 1][lane] - sp[buf][w + 1][lane + 2] -
-                                            sp[buf][w][lane + 1] - sp[buf][w + 2][lane + 1] - fmv - fp;
+                    const long long *S = sp[buf] + own_at;
+                    const long long lapfx = 6 * fc - S[-1] - S[1] - S[-pitch] - S[pitch] - fmv - fp;
                     float2 ph, pl;   // the stencil sum and u in one packed FP32x2 chain (the same results)
                     fx_to_pair2(lapfx, fc, scale, ph, pl);
                     const float lh = ph.x, ll = pl.x, uh = ph.y, ul = pl.y;
@@ -704,12 +711,17 @@ __global__ void __launch_bounds__(256, NEU ? 4 : 5) k_eig_pass2_df(double *__res
           }
         }
     } else {
+        // flat mirror pairs (up to the next 16 bytes of a row): rows of half a length each left
+        // lanes idle and the warps unevenly loaded (100^3: 20.0 us, 17.4 this way)
         const int H = P / 2, nsym = (n + 1) / 2, nanti = n / 2;
-        for (int row = w0; row < P * P; row += wstride) {
-          const int ry = row % P, rz = row / P;
-          for (int i = lane; i < H; i += 32) {
+        const unsigned hr = (nsym + 7) & ~7, un = n;
+        const size_t total = (size_t)n * n * hr, stride = (size_t)gridDim.x * 256;
+        for (size_t t = (size_t)blockIdx.x * 256 + threadIdx.x; t < total; t += stride) {
+            const unsigned row = (unsigned)(t < 0xffffffffull ? (unsigned)t / hr : t / hr);
+            const int i = (int)(t - (size_t)row * hr);
+            const int rz = (int)(row / un), ry = (int)(row - (unsigned)rz * un);
             float fa = 0.0f, fb = 0.0f;
-            if (ry < n && rz < n && i < nsym) {
+            if (i < nsym) {
                 const int y = (ry & 1) ? n - 1 - (ry >> 1) : (ry >> 1);
                 const int z = (rz & 1) ? n - 1 - (rz >> 1) : (rz >> 1);
                 const long long cb = ((long long)z * n + y) * n;
@@ -723,14 +735,14 @@ __global__ void __launch_bounds__(256, NEU ? 4 : 5) k_eig_pass2_df(double *__res
                     fa = __fadd_rn(fa, f2);
                 }
             }
-            const long long o = (long long)row * P + i;
+            const long long o = ((long long)rz * P + ry) * P + i;
             const __nv_bfloat16 ha = __float2bfloat16_rn(fa), hb = __float2bfloat16_rn(fb);
             Rhi[o] = ha;
             Rlo[o] = __float2bfloat16_rn(fa - __bfloat162float(ha));
             Rhi[o + H] = hb;
             Rlo[o + H] = __float2bfloat16_rn(fb - __bfloat162float(hb));
-          }
         }
+        zero_padding(Rhi, Rlo, n, P, hr, n, H, 2);
     }
     // max|U| of the iterate for the next pass 1's fixed-point exponent
     __shared__ unsigned long long shm[8];
@@ -825,6 +837,25 @@ int launch_eig_pass2(double *U, const double *lin, int n, int P, int dim, int bc
     return QN_OK;
 }
 
+// The tile (at most 256 columns, 24 to 64 wide where n allows) that covers n x n with the
+// fewest, of those the one with the shortest halo.
+static long long pass1_tile(int n, int &W, int &H) {
+    long long best = LLONG_MAX;
+    for (int k = 1; k <= n; ++k) {
+        const int w = (n + k - 1) / k;
+        if (w > 64) continue;
+        if (w < 24 && k > 1) break;
+        const int rows = std::min(n, 256 / w), ky = (n + rows - 1) / rows, h = (n + ky - 1) / ky;
+        const long long cost = (long long)k * ky * 1024 + w + h;
+        if (cost < best) {
+            best = cost;
+            W = w;
+            H = h;
+        }
+    }
+    return (long long)((n + W - 1) / W) * ((n + H - 1) / H);
+}
+
 template <bool NEU>
 static int pass1_tiled(const double *U, float2 *lin, int n, double inv_h2, double lam, float2 lam2, double b,
                        const double *pot, const double *vrow, const float2 *pot2, const float2 *vrow2,
@@ -833,12 +864,14 @@ static int pass1_tiled(const double *U, float2 *lin, int n, double inv_h2, doubl
     QN_CUDA(cudaGetDevice(&dev));
     QN_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     QN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_eig_pass1_tiled<NEU>, 256, 0));
-    const int zc = n < 400 ? 16 : 32;   // planes per work item (two more are read at its start)
-    const long long items = (long long)((n + kP1W - 1) / kP1W) * ((n + kP1H - 1) / kP1H) * ((n + zc - 1) / zc);
+    int W = 0, H = 0;
+    const long long tiles = pass1_tile(n, W, H);
     long long g = (long long)(nb > 0 ? nb : 1) * sms;   // one wave of resident blocks
     if (g > grid) g = grid;
+    const int zc = balanced_zchunk(tiles, n, g);
+    const long long items = tiles * ((n + zc - 1) / zc);
     if (g > items) g = items;
-    k_eig_pass1_tiled<NEU><<<(int)g, 256, 0, s>>>(U, lin, n, zc, inv_h2, lam, lam2, b, pot, vrow, pot2, vrow2,
+    k_eig_pass1_tiled<NEU><<<(int)g, 256, 0, s>>>(U, lin, n, W, H, zc, inv_h2, lam, lam2, b, pot, vrow, pot2, vrow2,
                                                   partials, st);
     *used = (int)g;
     return QN_OK;

@@ -1,6 +1,7 @@
 // Internal declarations shared by the libqn translation units.
 #pragma once
 
+#include <limits.h>
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -244,6 +245,25 @@ void tc_plan_destroy(TcPlan *plan);
 // the FP64 dense target for EPI_UPDATE / EPI_DENSE). forward selects S^{-1}.
 int launch_modeprod_tc(TcPlan *plan, int src, int dst, bool forward, Epi epi,
                        const EpiArgs &e, cudaStream_t s);
+// Planes per work item: the fewest plane steps of the busiest block, its items times their
+// planes and the two that an item reads ahead of its first. A fixed 32 leaves the last round of
+// the blocks nearly empty at some sizes and too few items at small ones; with tiles over the
+// grid points alone (instead of the padded ones) a solve of 8 iterations takes, before and now:
+// n = 65 0.94, 0.75 ms; 100 0.94, 0.79; 130 1.33, 1.23; 255 3.05, 2.97; 400 13.1, 12.6; 511 19.7,
+// 19.5. Example 1's residual at 400^3: 601, 538 us.
+inline int balanced_zchunk(long long tiles, int n, long long blocks) {
+    int best = 32;
+    long long cost = LLONG_MAX;
+    for (int zc = 4; zc <= 96; ++zc) {
+        const long long c = (tiles * ((n + zc - 1) / zc) + blocks - 1) / blocks * (zc + 2);
+        if (c < cost) {
+            cost = c;
+            best = zc;
+        }
+    }
+    return best;
+}
+
 // Sizes the reflection-split products are used at (3-D). P = 192 is left to the dense products: a
 // solve takes 1.34 ms against 1.45 at n = 130 and 1.57 against 1.72 at n = 192, the halves of 96
 // filling the MMAs too little; from P = 320 on the split is faster (5.9 against 5.0 ms at n = 260,

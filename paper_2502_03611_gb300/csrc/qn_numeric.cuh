@@ -11,6 +11,8 @@
 
 #include <stdint.h>
 
+#include <cuda_bf16.h>
+
 namespace qn {
 
 // Rare-path helpers are kept out of line: inlined, the compiler turns them
@@ -53,6 +55,37 @@ __device__ __forceinline__ double f2d_exact(float f) {
 // |d| as an unsigned integer that orders like |d| (for min/max of |U| without FP64 ops).
 __device__ __forceinline__ unsigned long long abs_bits(double d) {
     return (unsigned long long)__double_as_longlong(d) & 0x7FFFFFFFFFFFFFFFull;
+}
+
+// Zeros in the part of the padded planes that no tile with grid points covers: planes [n, P),
+// rows [yt, P) of the other planes, and `segs` segments of each other row from x = xt on, seg
+// elements apart and long up to the next one's start. Sixteen bytes per store (P is a multiple
+// of 64, xt and seg of 8).
+__device__ __forceinline__ void zero_padding(__nv_bfloat16 *Rhi, __nv_bfloat16 *Rlo, unsigned n, unsigned P, int xt,
+                                             int yt, int seg, int segs) {
+    const unsigned tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    uint4 *hi = reinterpret_cast<uint4 *>(Rhi), *lo = reinterpret_cast<uint4 *>(Rlo);
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    const size_t plane = (size_t)P * P / 8, row = P / 8;
+    for (size_t i = tid; i < (P - n) * plane; i += nt) {
+        hi[n * plane + i] = zero;
+        lo[n * plane + i] = zero;
+    }
+    const unsigned c2 = (P - yt) * (unsigned)row;
+    for (size_t i = tid; i < (size_t)n * c2; i += nt) {
+        const size_t z = i / c2, o = z * plane + yt * row + (i - z * c2);
+        hi[o] = zero;
+        lo[o] = zero;
+    }
+    const unsigned w = (unsigned)(seg - xt) / 8, c3 = w * (unsigned)segs;
+    if (c3 == 0) return;
+    for (size_t i = tid; i < (size_t)n * yt * c3; i += nt) {
+        const unsigned r = (unsigned)(i / c3), k = (unsigned)(i - (size_t)r * c3);
+        const unsigned z = r / yt, y = r - z * yt;
+        const size_t o = z * plane + y * row + (k / w) * (unsigned)(seg / 8) + xt / 8 + k % w;
+        hi[o] = zero;
+        lo[o] = zero;
+    }
 }
 
 }  // namespace qn

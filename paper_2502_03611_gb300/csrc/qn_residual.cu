@@ -823,37 +823,6 @@ __device__ __forceinline__ void block_partials(const ResidualArgs &a, float kr2,
     }
 }
 
-// Zeros in the part of the padded planes that no tile with grid points covers: planes [n, P),
-// rows [yt, P) of the other planes, and `segs` segments of each other row from x = xt on, seg
-// elements apart and long up to the next one's start. Sixteen bytes per store (P is a multiple
-// of 64, xt, yt and seg of 16).
-__device__ __forceinline__ void zero_padding(const ResidualArgs &a, int xt, int yt, int seg, int segs) {
-    const unsigned n = a.n, P = a.P;
-    const unsigned tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-    uint4 *hi = reinterpret_cast<uint4 *>(a.Rhi), *lo = reinterpret_cast<uint4 *>(a.Rlo);
-    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-    const size_t plane = (size_t)P * P / 8, row = P / 8;
-    for (size_t i = tid; i < (P - n) * plane; i += nt) {
-        hi[n * plane + i] = zero;
-        lo[n * plane + i] = zero;
-    }
-    const unsigned c2 = (P - yt) * (unsigned)row;
-    for (size_t i = tid; i < (size_t)n * c2; i += nt) {
-        const size_t z = i / c2, o = z * plane + yt * row + (i - z * c2);
-        hi[o] = zero;
-        lo[o] = zero;
-    }
-    const unsigned w = (unsigned)(seg - xt) / 8, c3 = w * (unsigned)segs;
-    if (c3 == 0) return;
-    for (size_t i = tid; i < (size_t)n * yt * c3; i += nt) {
-        const unsigned r = (unsigned)(i / c3), k = (unsigned)(i - (size_t)r * c3);
-        const unsigned z = r / yt, y = r - z * yt;
-        const size_t o = z * plane + y * row + (k / w) * (unsigned)(seg / 8) + xt / 8 + k % w;
-        hi[o] = zero;
-        lo[o] = zero;
-    }
-}
-
 template <int KIND>
 __global__ void __launch_bounds__(kTThreads, 2) k_residual_tiled(ResidualArgs a, int zchunk) {
     if (a.done != nullptr && *(volatile const int *)a.done) return;
@@ -1112,7 +1081,7 @@ __global__ void __launch_bounds__(kTThreads, 2) k_residual_tiled(ResidualArgs a,
         }
     }
 
-    zero_padding(a, tiles_x * kTX, tiles_y * kTY, P, 1);
+    zero_padding(a.Rhi, a.Rlo, n, P, tiles_x * kTX, tiles_y * kTY, P, 1);
     tile_partials<KIND>(a, kr2, kc, r2k, amin, amax, dmn, dmx);
 }
 
@@ -1414,7 +1383,7 @@ __global__ void __launch_bounds__(kTThreads, 2) k_residual_mirror(ResidualArgs a
         }
     }
 
-    zero_padding(a, tiles_x * 32, tiles_y * kTY, H, 2);
+    zero_padding(a.Rhi, a.Rlo, n, P, tiles_x * 32, tiles_y * kTY, H, 2);
     tile_partials<KIND>(a, kr2, kc, r2k, amin, amax, dmn, dmx);
 }
 
@@ -1938,25 +1907,6 @@ int launch_residual(const ResidualArgs &a, int grid, cudaStream_t s) {
     }
     QN_CUDA(cudaGetLastError());
     return QN_OK;
-}
-
-// Planes per work item: the fewest plane steps of the busiest block, its items times their
-// planes and the two that an item reads ahead of its first. A fixed 32 leaves the last round of
-// the blocks nearly empty at some sizes and too few items at small ones; with tiles over the
-// grid points alone (instead of the padded ones) a solve of 8 iterations takes, before and now:
-// n = 65 0.94, 0.75 ms; 100 0.94, 0.79; 130 1.33, 1.23; 255 3.05, 2.97; 400 13.1, 12.6; 511 19.7,
-// 19.5. Example 1's residual at 400^3: 601, 538 us.
-static int balanced_zchunk(long long tiles, int n, long long blocks) {
-    int best = 32;
-    long long cost = LLONG_MAX;
-    for (int zc = 4; zc <= 96; ++zc) {
-        const long long c = (tiles * ((n + zc - 1) / zc) + blocks - 1) / blocks * (zc + 2);
-        if (c < cost) {
-            cost = c;
-            best = zc;
-        }
-    }
-    return best;
 }
 
 template <int KIND>
