@@ -644,21 +644,22 @@ __global__ void __launch_bounds__(256, 3) k_eig_pass1_tiled(const double *__rest
     }
 }
 
-// One node of pass 2 in float pairs; U = s U~ written back (the one FP64 multiply).
+// One node of pass 2 in float pairs, u0 = U~ and lin0 read by the caller (a node's store would
+// hold back the next node's loads); U = s U~ written back (the one FP64 multiply).
 template <int DIM, bool NEU>
-__device__ __forceinline__ float eig_point_df(double *__restrict__ U, const float2 *__restrict__ lin, long long c,
+__device__ __forceinline__ float eig_point_df(double *__restrict__ U, double u0, float2 lin0, long long c,
                                               int x, int y, int z, int n, double sc, float2 sc2, float2 lamn2,
                                               float2 b2, float lamf, float b3f, const float *__restrict__ pot32,
                                               float &sk, float &kc, float &dmn, float &dmx,
                                               unsigned long long &umax) {
-    const double u = sc * U[c];
+    const double u = sc * u0;
     U[c] = u;
     const unsigned long long ab = abs_bits(u);
     umax = ab > umax ? ab : umax;
     const float2 up = f_pair(u, nullptr);
     const float2 u2 = pair_mul(up, up);
     const float2 bu3 = pair_mul(b2, pair_mul(u2, up));
-    const float2 F = pair_add(pair_add(pair_mul(sc2, __ldg(lin + c)), bu3), pair_neg(pair_mul(lamn2, up)));
+    const float2 F = pair_add(pair_add(pair_mul(sc2, lin0), bu3), pair_neg(pair_mul(lamn2, up)));
     const float Ff = __fadd_rn(F.x, F.y);
     float wF = Ff;
     if (NEU) wF = Ff * (float)(tw<NEU>(x, n) * tw<NEU>(y, n) * ((DIM == 3) ? tw<NEU>(z, n) : 1.0));
@@ -702,7 +703,7 @@ __global__ void __launch_bounds__(256, NEU ? 4 : 5) k_eig_pass2_df(double *__res
             float f = 0.0f;
             if (x < n && y < n && z < n) {
                 const long long c = ((long long)z * n + y) * n + x;
-                f = eig_point_df<DIM, NEU>(U, lin, c, x, y, z, n, sc, sc2, lamn2, b2, lamf, b3f, pot32, sk, kc, dmn,
+                f = eig_point_df<DIM, NEU>(U, U[c], __ldg(lin + c), c, x, y, z, n, sc, sc2, lamn2, b2, lamf, b3f, pot32, sk, kc, dmn,
                                            dmx, umax);
             }
             const __nv_bfloat16 hi = __float2bfloat16_rn(f);
@@ -712,7 +713,7 @@ __global__ void __launch_bounds__(256, NEU ? 4 : 5) k_eig_pass2_df(double *__res
         }
     } else {
         // flat mirror pairs (up to the next 16 bytes of a row): rows of half a length each left
-        // lanes idle and the warps unevenly loaded (100^3: 20.0 us, 17.4 this way)
+        // lanes idle and the warps unevenly loaded (100^3: 20.0 us, 17.4 this way, 16.2 with both nodes read first)
         const int H = P / 2, nsym = (n + 1) / 2, nanti = n / 2;
         const unsigned hr = (nsym + 7) & ~7, un = n;
         const size_t total = (size_t)n * n * hr, stride = (size_t)gridDim.x * 256;
@@ -725,11 +726,13 @@ __global__ void __launch_bounds__(256, NEU ? 4 : 5) k_eig_pass2_df(double *__res
                 const int y = (ry & 1) ? n - 1 - (ry >> 1) : (ry >> 1);
                 const int z = (rz & 1) ? n - 1 - (rz >> 1) : (rz >> 1);
                 const long long cb = ((long long)z * n + y) * n;
-                fa = eig_point_df<DIM, NEU>(U, lin, cb + i, i, y, z, n, sc, sc2, lamn2, b2, lamf, b3f, pot32, sk, kc,
+                const int j = n - 1 - i;   // (the node itself in the middle of an odd row)
+                const double ua = U[cb + i], ub = U[cb + j];
+                const float2 la = __ldg(lin + cb + i), lb = __ldg(lin + cb + j);
+                fa = eig_point_df<DIM, NEU>(U, ua, la, cb + i, i, y, z, n, sc, sc2, lamn2, b2, lamf, b3f, pot32, sk, kc,
                                             dmn, dmx, umax);
                 if (i < nanti) {
-                    const int j = n - 1 - i;
-                    const float f2 = eig_point_df<DIM, NEU>(U, lin, cb + j, j, y, z, n, sc, sc2, lamn2, b2, lamf, b3f,
+                    const float f2 = eig_point_df<DIM, NEU>(U, ub, lb, cb + j, j, y, z, n, sc, sc2, lamn2, b2, lamf, b3f,
                                                             pot32, sk, kc, dmn, dmx, umax);
                     fb = __fsub_rn(fa, f2);
                     fa = __fadd_rn(fa, f2);
