@@ -68,7 +68,10 @@ extern "C" {
                                qn_problem.robin_kappa >= 0 (the face term belongs to A_h);
                                finite differences, per-node residual kernel */
 
-#define QN_PREC_FP64   0    /* mode products in FP64 on the FP64 pipe */
+#define QN_PREC_FP64   0    /* mode products of FP64 operands with FP64 results: n^(dim+1) above
+                               6e6 as exact integer digits on the tensor cores (seven nine-bit
+                               digits per value, rounded at the end; closer to the exact product
+                               than a chain of FP64 multiply-adds), smaller ones on the FP64 pipe */
 #define QN_PREC_BF16X3 1    /* mode products on tcgen05 tensor cores as
                                hi*hi + hi*lo + lo*hi BF16 products, FP32
                                accumulation; residual, beta, update and stop
@@ -192,7 +195,8 @@ int qn_setup_1d_sem(int n, int k, double length, int bc, double *H, double *S, d
 /* Create a context for one problem shape on the current CUDA device: uploads
  * S, S^{-1} and the eigenvalues (and their BF16 hi/lo splits for
  * QN_PREC_BF16X3 / BF16X6), allocates the working buffers (about 2 n^dim doubles for
- * FP64, 2 padded n^dim x 4 bytes for BF16X3) and, for BF16X3, builds the TMA
+ * FP64, where the products run on the tensor cores with the digits of one operand besides:
+ * 14 bytes per value, at most 2 GiB at a time; 2 padded n^dim x 4 bytes for BF16X3) and, for BF16X3, builds the TMA
  * tensor maps. QN_EUNSUPPORTED for BF16X3 on a device without sm_103a
  * tcgen05 support. *out is owned by the library until qn_ctx_destroy. */
 int qn_ctx_create(const qn_problem *p, qn_ctx **out);
@@ -262,7 +266,8 @@ int qn_set_escalation(qn_ctx *ctx, double rate);
  * kernel and product. The iterates are those of the separate kernels: the same fixed-point
  * stencil, float-pair nonlinear term and products; only the FP32 summation order of
  * ||F||^2 differs. QN_EUNSUPPORTED (on != 0) unless the context is a 3-D BF16X3 or
- * BF16X6 finite-difference context with the reflection-split products, n <= 512,
+ * BF16X6 finite-difference context with the reflection-split products, n <= 512 and
+ * P = 64 ceil(n/64) a multiple of 128,
  * Dirichlet data and no potential. The first call with on != 0 encodes two tensor maps
  * (a blocking copy to the device): call it outside a stream capture. Does not
  * synchronise otherwise. qn_profile.fused_launches / fused_ms time the fused kernel.
@@ -506,8 +511,8 @@ typedef struct qn_profile {
                                       from its third iteration on (no FP64 arithmetic) */
     double residual_tiled_ms;
     int split_products;       /* 1: the last shifted inverse used the reflection-split mode
-                                 products (3-D split solve, n+ padding a multiple of 128):
-                                 half the tensor work of the dense products */
+                                 products (3-D split solve; P = 64 ceil(n/64) a multiple of
+                                 128, or at least 320): half the tensor work of the dense products */
     int x6_from;              /* the last qn_solve: the first iteration whose backward products
                                  ran at the six-product level (0 in a QN_PREC_BF16X6 context,
                                  the escalation point after qn_set_escalation), -1: none */
