@@ -46,7 +46,8 @@ namespace qn {
 namespace {
 
 constexpr int kDig = 7;                  // digits per value
-constexpr int BM = 128, BK = 32;         // tile rows; K per pipeline stage (a 64-byte swizzle row)
+constexpr int BM = 128, BK = 64;         // tile rows; K per pipeline step (a 128-byte swizzle row)
+constexpr int kSlots = 9;                // digit tiles of A and B in shared memory
 constexpr int kSegK = 128;               // terms per accumulator
 constexpr int kTotal = 256;              // terms whose 64-bit sum fits with full-range digits
 constexpr int kEpiWarps = 16;            // four warps per TMEM lane quadrant
@@ -259,7 +260,7 @@ __device__ __forceinline__ double scaled(long long v, int e) {
 __device__ __noinline__ double divided_slow(long long v, int e, double d) { return scalbn((double)v, e) / d; }
 
 // integer * 2^e / d. The FP64 pipe would need about nine of its slow operations per output for
-// the division (415 us for a 255^3 product, against 136 us without it and 163 us this way), so the quotient is
+// the division (415 us for a 255^3 product, against 144 us without it), so the quotient is
 // formed on the integer pipe: a reciprocal of the divisor's 64-bit significand from an FP32
 // seed and two terms of the series 1/d = x (1 + e + e^2 + ..), e = 1 - d x, |e| < 2^-22, good to
 // about 2^-60, times the normalised integer; rounded to 53 bits once.
@@ -329,43 +330,47 @@ __device__ __forceinline__ void tmem_ld(uint32_t addr, uint32_t (&r)[NC]) {
 }
 
 template <int BN>
-__host__ __device__ constexpr uint32_t stage_bytes() {
-    return kDig * (BM + BN) * BK * 2;
+__host__ __device__ constexpr uint32_t slot_bytes() {
+    return (BM + BN) * BK * 2;
 }
 
-__host__ __device__ constexpr int stages_for(int BN) {
-    return (int)((227 * 1024 - 1024 - kCtrlBytes) / (kDig * (BM + BN) * BK * 2));
+// The order in which the seven digit tiles of a K step are released. Tile t of a step (digit t
+// of A and of B) is multiplied with the tiles j <= min(t, 6 - t) that came before it, so tile i
+// is last used at t = max(i, 6 - i), and a commit after those MMAs releases its slot. With nine
+// slots, tiles 0 and 1 of the next step load into the spare two, its tiles 2..6 into the slots
+// released first, and tiles 0 and 6 of this step are the next spare ones. A step's slots are packed
+// four bits each.
+__device__ __forceinline__ uint32_t next_slots(uint32_t prev2, uint32_t prev1) {
+    auto at = [](uint32_t m, int t) { return (m >> (4 * t)) & 15u; };
+    return at(prev2, 0) | at(prev2, 6) << 4 | at(prev1, 3) << 8 | at(prev1, 2) << 12 | at(prev1, 4) << 16 |
+           at(prev1, 1) << 20 | at(prev1, 5) << 24;
 }
+constexpr uint32_t kSlots0 = 0x6543210u, kSlotsBefore = 0x8000007u;
 
 // Persistent, one CTA of 576 threads per SM: warp 0 loads the digit tiles by TMA, warp 1 issues
-// the MMAs, warps 2..17 are the epilogue. A stage holds the seven digits of 128 x 32 of A and
-// BN x 32 of B (84 KB at BN = 64, two stages). For every K = 16 step the seven A digits are
-// copied to tensor memory (tcgen05.cp, 56 columns beside the accumulators), because each is used
-// by up to seven MMAs: an M = 128, K = 16 MMA of 16 to 64 columns takes 37 to 46 clocks with A in
-// shared memory, which it reads whole each time, and 9 to 30 with A in tensor memory. An
-// inverse at 255^3 goes from 1370 to 1264 us, at 200^3 from 894 to 853, at 383^3 from 5716 to
-// 5169; 255^2 and 64^3 stay at 98 and 111 us. Separate rings for A and B, with B kept across
-// the row tiles, were slower (1290 us).
+// the MMAs, warps 2..17 are the epilogue. TMEM holds seven accumulators of BN columns (448 of
+// 512 at BN = 64), so they are not double-buffered as a whole; each has its own full / empty
+// barrier instead. Taking the digits in order makes accumulator d complete with tile d of the
+// last K step and first needed again with tile ceil(d/2) of the next sum, so the epilogue
+// drains them in order d = 0..6 while the MMAs run on.
 //
-// TMEM holds seven accumulators of BN columns (448 of 512 at BN = 64), so they are not
-// double-buffered as a whole; each has its own full / empty barrier instead. The MMAs run in
-// the order of d, so accumulator d is complete before those of d + 1 in the last K step and
-// first needed again after those of d - 1 in the next sum: the epilogue drains them in order
-// d = 0..6 while the MMAs run on.
+// A in tensor memory (tcgen05.cp of the seven digits per K = 16 step, where an MMA does not read
+// 128 rows of shared memory each time) needs the readers of those columns to be done before the
+// next copy: copies are ordered before later MMAs, not after earlier ones. An inverse at 255^3
+// takes 1370 us as it is; with the waits and one set of columns in two groups 1419, eight slots
+// in turn 1447, tiles of 48 columns and three sets 1634, of 32 and four sets 1899.
 template <int BN, int MODE, int EPI>
 __global__ void __maxnreg__(96) k_modeprod_f64tc(const ProdArgs g) {
     if (g.e.done != nullptr && *(volatile const int *)g.e.done) return;
-    constexpr uint32_t a_dig = BM * BK * 2, b_dig = BN * BK * 2;
-    constexpr uint32_t kStage = stage_bytes<BN>();
-    constexpr int kStages = stages_for(BN);
+    constexpr uint32_t a_bytes = BM * BK * 2;
+    constexpr uint32_t kSlot = slot_bytes<BN>();
     constexpr int NC = BN / (kEpiWarps / 4);   // columns per epilogue thread
-    constexpr uint32_t kACol = kDig * BN;      // A digits of one K = 16 step: 7 x 8 columns
-    static_assert(kACol + kDig * 8 <= 512 && kStages >= 2 && kStages <= 4, "TMEM columns, stages");
+    static_assert(kDig * BN <= 512, "TMEM columns");
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = ptx::smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
-    const uint32_t ctrl = base + kStages * kStage;
+    const uint32_t ctrl = base + kSlots * kSlot;
     auto full_bar = [&](uint32_t s) { return ctrl + 8u * s; };
     auto empty_bar = [&](uint32_t s) { return ctrl + 80u + 8u * s; };
     auto tfull_bar = [&](int d) { return ctrl + 160u + 8u * d; };
@@ -376,7 +381,7 @@ __global__ void __maxnreg__(96) k_modeprod_f64tc(const ProdArgs g) {
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) {
+        for (int s = 0; s < kSlots; ++s) {
             ptx::mbar_init(full_bar(s), 1);
             ptx::mbar_init(empty_bar(s), 1);
         }
@@ -407,40 +412,42 @@ __global__ void __maxnreg__(96) k_modeprod_f64tc(const ProdArgs g) {
     const int nseg = (steps + kSegSteps - 1) / kSegSteps;
 
     if (warp == 0 && lane == 0) {
-        uint32_t armed_parity[kStages], armed = 0, ph = 0;
-        int s = 0;
+        uint32_t phase = 0, armed = 0;   // per slot: the next load's phase; loaded at least once
+        uint32_t sl1 = kSlotsBefore, sl = kSlots0;
         bool ok = true;
         for (int t = blockIdx.x; ok && t < g.ntiles; t += gridDim.x) {
             const int mt = t / tpm, r = t % tpm;
             const int n0 = (r % g.ntn) * BN;
             const int x0 = (MODE == MD_FWD) ? (r / g.ntn) * g.Kp : 0;
-            for (int k = 0; k < kHalves * steps; ++k) {
-                if (!ptx::wait_bar(empty_bar(s), ph ^ 1u, abort_flag, g.e.err)) {
-                    ok = false;
-                    break;
+            for (int k = 0; ok && k < kHalves * steps; ++k) {
+                for (int d = 0; d < kDig; ++d) {
+                    const uint32_t s = (sl >> (4 * d)) & 15u;
+                    if (!ptx::wait_bar(empty_bar(s), ((phase >> s) & 1u) ^ 1u, abort_flag, g.e.err)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t st = base + s * kSlot;
+                    ptx::mbar_arrive_expect_tx(full_bar(s), kSlot);
+                    ptx::tma_load_3d(st, g.amap, full_bar(s), x0 + k * BK, mt * BM, d);
+                    ptx::tma_load_3d(st + a_bytes, g.bmap, full_bar(s), x0 + k * BK, n0, d);
+                    phase ^= 1u << s;
+                    armed |= 1u << s;
                 }
-                const uint32_t st = base + (uint32_t)s * kStage;
-                ptx::mbar_arrive_expect_tx(full_bar(s), kStage);
-                ptx::tma_load_3d(st, g.amap, full_bar(s), x0 + k * BK, mt * BM, 0);
-                ptx::tma_load_3d(st + kDig * a_dig, g.bmap, full_bar(s), x0 + k * BK, n0, 0);
-                armed_parity[s] = ph;
-                armed |= 1u << s;
-                if (++s == kStages) {
-                    s = 0;
-                    ph ^= 1u;
-                }
+                const uint32_t nx = next_slots(sl1, sl);
+                sl1 = sl;
+                sl = nx;
             }
         }
         if (!ok)
-            for (int i = 0; i < kStages; ++i)
-                if (armed & (1u << i)) ptx::drain_bar(full_bar(i), armed_parity[i]);
+            for (int i = 0; i < kSlots; ++i)
+                if (armed & (1u << i)) ptx::drain_bar(full_bar(i), ((phase >> i) & 1u) ^ 1u);
     } else if (warp == 1) {
         constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((BM >> 4) << 24);   // FP16, FP32 sums
         auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
             return __all_sync(0xffffffffu, ptx::wait_bar(bar, parity, abort_flag, g.e.err));
         };
-        uint32_t ph = 0, tp = 0;
-        int s = 0;
+        uint32_t phase = 0, tp = 0;
+        uint32_t sl1 = kSlotsBefore, sl = kSlots0;
         bool ok = true;
         for (int t = blockIdx.x; ok && t < g.ntiles; t += gridDim.x) {
             for (int step = 0; ok && step < kHalves * steps; ++step) {
@@ -448,46 +455,49 @@ __global__ void __maxnreg__(96) k_modeprod_f64tc(const ProdArgs g) {
                 const bool first = hs % kSegSteps == 0;
                 const bool last = hs % kSegSteps == kSegSteps - 1 || hs == steps - 1;
                 const int nk = min(BK, g.Kt - hs * BK) / 16;   // K = 16 MMAs of this step
-                ok = wait(full_bar(s), ph);
-                if (!ok) break;
-                ptx::tc_fence_after();
-                const uint32_t st = base + (uint32_t)s * kStage;
-                const uint64_t da = ptx::smem_desc_kmajor(st, BK * 2, 4);
-                const uint64_t db = ptx::smem_desc_kmajor(st + kDig * a_dig, BK * 2, 4);
-                for (int kk = 0; kk < nk; ++kk) {
-                    const bool end = last && kk == nk - 1;
-                    if (ptx::elect_one()) {
+                uint64_t da[kDig], db[kDig];
 #pragma unroll
-                        for (int i = 0; i < kDig; ++i)
-                            ptx::tmem_cp_128x256b(tmem_base + kACol + 8 * i, da + (i * a_dig) / 16 + 2 * kk);
-                    }
-                    __syncwarp();
+                for (int i = 0; i < kDig; ++i) {
+                    const uint32_t st = base + ((sl >> (4 * i)) & 15u) * kSlot;
+                    da[i] = ptx::smem_desc_kmajor(st, BK * 2, 2);
+                    db[i] = ptx::smem_desc_kmajor(st + a_bytes, BK * 2, 2);
+                }
 #pragma unroll
-                    for (int d = 0; d < kDig; ++d) {
-                        if (first && kk == 0) {
-                            ok = ok && wait(tempty_bar(d), tp ^ 1u);
-                            if (!ok) break;
-                            ptx::tc_fence_after();
-                        }
-                        if (ptx::elect_one()) {
-#pragma unroll
-                            for (int i = 0; i <= d; ++i)
-                                ptx::mma_f16_ts(tmem_base + (uint32_t)(d * BN), tmem_base + kACol + 8 * i,
-                                                db + ((d - i) * b_dig) / 16 + 2 * kk, idesc,
-                                                (i == 0 && first && kk == 0) ? 0u : 1u);
-                            if (end) ptx::mma_commit(tfull_bar(d));
-                        }
-                        __syncwarp();
+                for (int i = 0; i < kDig; ++i) {
+                    const uint32_t s = (sl >> (4 * i)) & 15u;
+                    if (ok) ok = wait(full_bar(s), (phase >> s) & 1u);
+                    phase ^= 1u << s;
+                    if (first && i <= 3) {   // accumulators 2i - 1 and 2i start with this tile
+                        if (ok && i > 0) ok = wait(tempty_bar(2 * i - 1), tp ^ 1u);
+                        if (ok) ok = wait(tempty_bar(2 * i), tp ^ 1u);
                     }
                     if (!ok) break;
-                }
-                if (ptx::elect_one()) ptx::mma_commit(empty_bar(s));
-                __syncwarp();
-                if (++s == kStages) {
-                    s = 0;
-                    ph ^= 1u;
+                    ptx::tc_fence_after();
+                    constexpr int jmax[kDig] = {0, 1, 2, 3, 2, 1, 0};   // min(i, 6 - i)
+                    if (ptx::elect_one()) {
+#pragma unroll
+                        for (int kk = 0; kk < BK / 16; ++kk) {
+                            if (kk >= nk) break;
+#pragma unroll
+                            for (int j = 0; j <= jmax[i]; ++j) {
+                                const uint32_t acc = tmem_base + (uint32_t)((i + j) * BN);
+                                // the first product into accumulator i + j overwrites it
+                                const uint32_t keep = (kk == 0 && i == (i + j + 1) / 2) ? (first ? 0u : 1u) : 1u;
+                                ptx::mma_f16(acc, da[i] + 2 * kk, db[j] + 2 * kk, idesc, keep);
+                                if (j != i) ptx::mma_f16(acc, da[j] + 2 * kk, db[i] + 2 * kk, idesc, 1u);
+                            }
+                        }
+                        if (last) ptx::mma_commit(tfull_bar(i));
+                        // tiles released by this one (see next_slots)
+                        if (i >= 3) ptx::mma_commit(empty_bar(s));
+                        if (i > 3) ptx::mma_commit(empty_bar((sl >> (4 * (6 - i))) & 15u));
+                    }
+                    __syncwarp();
                 }
                 if (last) tp ^= 1u;
+                const uint32_t nx = next_slots(sl1, sl);
+                sl1 = sl;
+                sl = nx;
             }
         }
         if (ptx::elect_one()) ptx::mma_commit(mma_done_bar);
@@ -597,7 +607,7 @@ __global__ void __maxnreg__(96) k_modeprod_f64tc(const ProdArgs g) {
     }
 }
 
-size_t smem_for(int BN) { return 1024 + (size_t)stages_for(BN) * kDig * (BM + BN) * BK * 2 + kCtrlBytes; }
+size_t smem_for(int BN) { return 1024 + (size_t)kSlots * (BM + BN) * BK * 2 + kCtrlBytes; }
 
 template <int KIND>
 int slice_kind(const SliceArgs &a, cudaStream_t s) {
@@ -664,12 +674,12 @@ int opt_in_bn() {
     return rc;
 }
 
-// Digits [kDig][rows][ld] as a 3-D FP16 tensor read in 32 x box_rows boxes of all digits.
+// Digits [kDig][rows][ld] as a 3-D FP16 tensor read in 64 x box_rows boxes of one digit.
 int encode_digits(CUtensorMap *m, const __half *ptr, int ld, int rows, int box_rows) {
     cuuint64_t dims[3] = {(cuuint64_t)ld, (cuuint64_t)rows, (cuuint64_t)kDig};
     cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)rows * ld * 2};
-    cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)box_rows, (cuuint32_t)kDig};
-    return tc_encode_tiled(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, ptr, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B);
+    cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)box_rows, 1};
+    return tc_encode_tiled(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, ptr, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
 }  // namespace

@@ -154,25 +154,6 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_
     mma_bf16(d_tmem, adesc, bdesc, idesc, accumulate);
 }
 
-// A from tensor memory (lane = row, eight 32-bit columns of FP16 pairs for K = 16).
-__device__ __forceinline__ void mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
-                                           uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-// 128 rows x 32 bytes from shared memory (matrix descriptor) to eight columns of tensor memory.
-// Copies and MMAs of one thread run in the order of issue (block-scaled MMA loops refill their one
-// set of scale columns the same way): MMAs issued later see the copy, earlier ones are not
-// disturbed by it.
-__device__ __forceinline__ void tmem_cp_128x256b(uint32_t taddr, uint64_t sdesc) {
-    asm volatile("tcgen05.cp.cta_group::1.128x256b [%0], %1;" ::"r"(taddr), "l"(sdesc) : "memory");
-}
-
 // True in one lane of the (converged) warp. Branching on it, with the control flow around it
 // warp-uniform, lets the compiler keep the operands of the tcgen05 instructions inside in
 // uniform registers; after a branch on the lane index it handles every lane on its own.
