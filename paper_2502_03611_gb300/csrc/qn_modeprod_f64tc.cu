@@ -14,11 +14,13 @@
 //      integers. The mirror sums and differences of the reflection split are formed there,
 //      exactly, on the integers.
 //   2. k_modeprod_f64tc forms the digit products D_i G_j with i + j <= 6 (28 tcgen05 products,
-//      FP16 operands, FP32 accumulation) into one TMEM accumulator per d = i + j, over at
-//      most kSegK = 128 terms at a time. A product of two digits is an integer of at most
-//      2^16, and the digits of B other than the leading one average half their range, so a
-//      sum of d + 1 products stays within 2^24, where FP32 sums of integers are exact, up to
-//      d = 3 whatever A holds; a rounding at d >= 4 would be 2^-52 of the largest product.
+//      FP16 operands, FP32 accumulation) into one TMEM accumulator per d = i + j. A product of
+//      two digits is an integer of at most 2^16, and FP32 sums of integers are exact up to 2^24 =
+//      256 products: accumulators 0 and 1 take kSegK = 128 terms at a time, 2 to 4 take
+//      BK = 64. So the sums up to d = 3 are exact whatever the digits. Those of d = 4 are while the
+//      five products of a term average below 0.8 of their range (a row of B that is constant may have
+//      more); a rounding there is 2^-51 of the largest product, within what a chain of FP64
+//      multiply-adds may lose on the same terms. d = 5 and 6 lie below the last bit that is kept.
 //   3. Its epilogue adds the seven accumulators as one 64-bit integer
 //      sum_d C_d 2^(38-9d), forms p +- q of the reflection split on the integers, converts
 //      once to FP64, applies the row's and the column's exponents and stores, divides or
@@ -48,7 +50,8 @@ namespace {
 constexpr int kDig = 7;                  // digits per value
 constexpr int BM = 128, BK = 64;         // tile rows; K per pipeline step (a 128-byte swizzle row)
 constexpr int kSlots = 9;                // digit tiles of A and B in shared memory
-constexpr int kSegK = 128;               // terms per accumulator
+constexpr int kSegK = 128;               // terms per sum of digit products,
+constexpr int kMid0 = 2, kMid1 = 4;      // of which these accumulators take BK at a time
 constexpr int kTotal = 256;              // terms whose 64-bit sum fits with full-range digits
 constexpr int kEpiWarps = 16;            // four warps per TMEM lane quadrant
 constexpr int kThreads = 64 + 32 * kEpiWarps;
@@ -356,9 +359,10 @@ constexpr uint32_t kSlots0 = 0x6543210u, kSlotsBefore = 0x8000007u;
 //
 // A in tensor memory (tcgen05.cp of the seven digits per K = 16 step, where an MMA does not read
 // 128 rows of shared memory each time) needs the readers of those columns to be done before the
-// next copy: copies are ordered before later MMAs, not after earlier ones. An inverse at 255^3
-// takes 1370 us as it is; with the waits and one set of columns in two groups 1419, eight slots
-// in turn 1447, tiles of 48 columns and three sets 1634, of 32 and four sets 1899.
+// next copy: copies are ordered before later MMAs, not after earlier ones. An inverse at 255^3,
+// with sums of 128 terms in every accumulator, took 1370 us as it is, with the waits and one set of
+// columns in two groups 1419, eight slots in turn 1447, tiles of 48 columns and three sets 1634,
+// of 32 and four sets 1899. (Emptying accumulators 2 to 4 every 64 terms takes 1370 to 1448.)
 template <int BN, int MODE, int EPI>
 __global__ void __maxnreg__(96) k_modeprod_f64tc(const ProdArgs g) {
     if (g.e.done != nullptr && *(volatile const int *)g.e.done) return;
@@ -405,11 +409,12 @@ __global__ void __maxnreg__(96) k_modeprod_f64tc(const ProdArgs g) {
     ptx::tc_fence_after();
     const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t *>(smem_raw + (tmem_slot - raw));
 
+    auto mid = [](int d) { return d >= kMid0 && d <= kMid1; };   // accumulators emptied every K step
     constexpr int kHalves = (MODE == MD_BWD) ? 2 : 1;   // halves summed by one tile
     const int tpm = (MODE == MD_FWD ? 2 : 1) * g.ntn;   // tiles per 128 rows
     const int steps = g.Kp / BK;                        // K steps of a half
     constexpr int kSegSteps = kSegK / BK;
-    const int nseg = (steps + kSegSteps - 1) / kSegSteps;
+    static_assert(2 * kSegK <= 256 && (kMid1) * BK <= 256, "digit sums within 2^24 up to d = 3");
 
     if (warp == 0 && lane == 0) {
         uint32_t phase = 0, armed = 0;   // per slot: the next load's phase; loaded at least once
@@ -446,7 +451,7 @@ __global__ void __maxnreg__(96) k_modeprod_f64tc(const ProdArgs g) {
         auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
             return __all_sync(0xffffffffu, ptx::wait_bar(bar, parity, abort_flag, g.e.err));
         };
-        uint32_t phase = 0, tp = 0;
+        uint32_t phase = 0, tp = 0, tm = 0;
         uint32_t sl1 = kSlotsBefore, sl = kSlots0;
         bool ok = true;
         for (int t = blockIdx.x; ok && t < g.ntiles; t += gridDim.x) {
@@ -467,10 +472,9 @@ __global__ void __maxnreg__(96) k_modeprod_f64tc(const ProdArgs g) {
                     const uint32_t s = (sl >> (4 * i)) & 15u;
                     if (ok) ok = wait(full_bar(s), (phase >> s) & 1u);
                     phase ^= 1u << s;
-                    if (first && i <= 3) {   // accumulators 2i - 1 and 2i start with this tile
-                        if (ok && i > 0) ok = wait(tempty_bar(2 * i - 1), tp ^ 1u);
-                        if (ok) ok = wait(tempty_bar(2 * i), tp ^ 1u);
-                    }
+#pragma unroll
+                    for (int d = 2 * i - 1; d <= 2 * i && i <= 3; ++d)   // these start with this tile
+                        if (ok && d >= 0 && (first || mid(d))) ok = wait(tempty_bar(d), (mid(d) ? tm : tp) ^ 1u);
                     if (!ok) break;
                     ptx::tc_fence_after();
                     constexpr int jmax[kDig] = {0, 1, 2, 3, 2, 1, 0};   // min(i, 6 - i)
@@ -482,12 +486,13 @@ __global__ void __maxnreg__(96) k_modeprod_f64tc(const ProdArgs g) {
                             for (int j = 0; j <= jmax[i]; ++j) {
                                 const uint32_t acc = tmem_base + (uint32_t)((i + j) * BN);
                                 // the first product into accumulator i + j overwrites it
-                                const uint32_t keep = (kk == 0 && i == (i + j + 1) / 2) ? (first ? 0u : 1u) : 1u;
+                                const uint32_t keep =
+                                    (kk == 0 && i == (i + j + 1) / 2) ? (first || mid(i + j) ? 0u : 1u) : 1u;
                                 ptx::mma_f16(acc, da[i] + 2 * kk, db[j] + 2 * kk, idesc, keep);
                                 if (j != i) ptx::mma_f16(acc, da[j] + 2 * kk, db[i] + 2 * kk, idesc, 1u);
                             }
                         }
-                        if (last) ptx::mma_commit(tfull_bar(i));
+                        if (last || mid(i)) ptx::mma_commit(tfull_bar(i));
                         // tiles released by this one (see next_slots)
                         if (i >= 3) ptx::mma_commit(empty_bar(s));
                         if (i > 3) ptx::mma_commit(empty_bar((sl >> (4 * (6 - i))) & 15u));
@@ -495,6 +500,7 @@ __global__ void __maxnreg__(96) k_modeprod_f64tc(const ProdArgs g) {
                     __syncwarp();
                 }
                 if (last) tp ^= 1u;
+                tm ^= 1u;
                 const uint32_t nx = next_slots(sl1, sl);
                 sl1 = sl;
                 sl = nx;
@@ -507,34 +513,38 @@ __global__ void __maxnreg__(96) k_modeprod_f64tc(const ProdArgs g) {
         const int quad = warp & 3, part = (warp - 2) >> 2;
         const int row = quad * 32 + lane;
         const uint32_t tcol = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(part * NC);
-        uint32_t tp = 0;
+        uint32_t tp = 0, tm = 0;
         bool ok = true;
-        // acc += sum_d C_d 2^(38-9d) of the next sum; false after a timeout (warp-uniform)
-        auto drain_sum = [&](long long(&acc)[NC]) -> bool {
+        // acc += sum_d C_d 2^(38-9d) of the next sum of `sub` K steps; false after a timeout (warp-uniform)
+        auto drain_sum = [&](long long(&acc)[NC], int sub) -> bool {
             float c5[NC];
+            for (int u = 1; u <= sub; ++u) {
 #pragma unroll
-            for (int d = 0; d < kDig; ++d) {
-                const bool ready = ptx::wait_bar(tfull_bar(d), tp, abort_flag, g.e.err);
-                if (!__all_sync(0xffffffffu, ready)) return false;
-                ptx::tc_fence_after();
-                uint32_t r[NC];
-                tmem_ld<NC>(tcol + (uint32_t)(d * BN), r);
-                ptx::tmem_ld_wait();
-                ptx::tc_fence_before();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(tempty_bar(d));
+                for (int d = 0; d < kDig; ++d) {
+                    if (u < sub && !mid(d)) continue;
+                    const bool ready = ptx::wait_bar(tfull_bar(d), mid(d) ? tm : tp, abort_flag, g.e.err);
+                    if (!__all_sync(0xffffffffu, ready)) return false;
+                    ptx::tc_fence_after();
+                    uint32_t r[NC];
+                    tmem_ld<NC>(tcol + (uint32_t)(d * BN), r);
+                    ptx::tmem_ld_wait();
+                    ptx::tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(tempty_bar(d));
 #pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    const float v = __uint_as_float(r[c]);
-                    if (d == 0)
-                        acc[c] += (long long)((unsigned long long)(unsigned)__float2int_rn(v) << 38);
-                    else if (d < 5)
-                        acc[c] = mad_wide(__float2int_rn(v), 1 << (38 - kBits * d), acc[c]);
-                    else if (d == 5)
-                        c5[c] = v;
-                    else
-                        acc[c] += (long long)__float2int_rn(fmaf(v, 0x1p-9f, c5[c]) * 0x1p-7f);
+                    for (int c = 0; c < NC; ++c) {
+                        const float v = __uint_as_float(r[c]);
+                        if (d == 0)
+                            acc[c] += (long long)((unsigned long long)(unsigned)__float2int_rn(v) << 38);
+                        else if (d < 5)
+                            acc[c] = mad_wide(__float2int_rn(v), 1 << (38 - kBits * d), acc[c]);
+                        else if (d == 5)
+                            c5[c] = v;
+                        else
+                            acc[c] += (long long)__float2int_rn(fmaf(v, 0x1p-9f, c5[c]) * 0x1p-7f);
+                    }
                 }
+                tm ^= 1u;
             }
             tp ^= 1u;
             return true;
@@ -546,11 +556,11 @@ __global__ void __maxnreg__(96) k_modeprod_f64tc(const ProdArgs g) {
             long long p[NC], q[(MODE == MD_BWD) ? NC : 1];
 #pragma unroll
             for (int c = 0; c < NC; ++c) p[c] = 0;
-            for (int seg = 0; ok && seg < nseg; ++seg) ok = drain_sum(p);
+            for (int at = 0; ok && at < steps; at += kSegSteps) ok = drain_sum(p, min(kSegSteps, steps - at));
             if constexpr (MODE == MD_BWD) {
 #pragma unroll
                 for (int c = 0; c < NC; ++c) q[c] = 0;
-                for (int seg = 0; ok && seg < nseg; ++seg) ok = drain_sum(q);
+                for (int at = 0; ok && at < steps; at += kSegSteps) ok = drain_sum(q, min(kSegSteps, steps - at));
             }
             if (!ok) break;
             const int ml = mt * BM + row;

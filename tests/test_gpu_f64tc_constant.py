@@ -1,0 +1,42 @@
+"""FP64 digit products whose digits repeat in every term: the constant row of the Neumann basis on
+fields that are constant up to 1e-7, where a sum of d + 1 digit products grows with the number of
+terms instead of averaging out. The inverse keeps the bound of any other field: 2 d products, each
+within 4 sqrt(n) roundings of its largest terms.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+# halves of 92, 128, 138, 188 and 256 terms; a dense basis with a constant row (Neumann spectral elements, n = 2 E + 1)
+@pytest.mark.parametrize("dim,n,sem", [(2, 183, 0), (2, 255, 0), (2, 275, 0), (2, 376, 0), (2, 511, 0), (3, 75, 0),
+                                       (2, 255, 2)])
+@pytest.mark.parametrize("rows", ["one constant", "one constant each"])
+def test_near_constant_fields(dim, n, sem, rows):
+    import torch
+
+    from paper_2502_03611_gb300 import qn
+    qn.load_library()
+    if sem:
+        _, S, Si, lam, _ = qn.qn_setup_1d_sem(n, sem, 1.0, qn.QN_BC_NEUMANN)
+        ctx = qn.QnContext(dim, n, "fp64", bc="neumann", sem_k=sem)
+    else:
+        S, Si, lam = qn.qn_setup_1d_eig(n, 1.0 / (n - 1), qn.QN_BC_NEUMANN)
+        ctx = qn.QnContext(dim, n, "fp64", bc="neumann")
+    rng = np.random.default_rng(n)
+    noise = 1.0 + 1e-7 * rng.standard_normal((n,) * dim)
+    cs = [0.96668, 0.7071, 0.5557, 0.9999] if rows == "one constant" else [None]
+    for c in cs:
+        r = noise * (c if c is not None else rng.uniform(0.5, 1.0, size=(n,) * (dim - 1) + (1,)))
+        t = torch.from_numpy(r).cuda()
+        V = torch.empty_like(t)
+        qn.qn_fast_diag_solve(ctx, t, V, 7.0)
+        X = r
+        for M in (Si, S):
+            for a in range(dim):
+                X = np.moveaxis(np.tensordot(M, X, axes=([1], [a])), 0, a)
+            if M is Si:
+                X = X / (sum(lam.reshape([-1 if a == b else 1 for b in range(dim)]) for a in range(dim)) + 7.0)
+        err = float(np.abs(V.cpu().numpy() - X).max() / np.abs(X).max())
+        assert err <= 2 * dim * 4.0 * np.sqrt(n) * 2.0 ** -52, (c, err)
