@@ -378,6 +378,8 @@ int launch_small_solve(const SmallSolve &q, cudaStream_t s) {
     if (grid < 1) grid = 1;
     if (grid > q.partials_cap) grid = q.partials_cap;
     if (grid < 1) grid = 1;
+    // a block holds both half matrices and its rows of U: one block's rows do not fit above n = 117
+    if (small_smem(q.n, grid) > 220 * 1024 && q.num_sms > 1 && q.partials_cap > 1) grid = 2;
     if (small_smem(q.n, grid) > 220 * 1024) {
         set_error("launch_small_solve: %d rows of n = %d per block do not fit in shared memory", (q.n + grid - 1) / grid,
                   q.n);
