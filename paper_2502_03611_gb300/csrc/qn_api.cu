@@ -541,14 +541,15 @@ extern "C" int qn_ctx_create(const qn_problem *p, qn_ctx **out) {
         CK(cudaMemcpy(c->hlen, len.data(), sizeof(int) * n, cudaMemcpyHostToDevice));
         CK(cudaMemcpy(c->hval, hv.data(), sizeof(double) * (size_t)n * bw, cudaMemcpyHostToDevice));
         if (p->precision != QN_PREC_FP64) {
-            // integers H 2^q, q such that every row sums to at most 2^58 in magnitude
+            // integers H 2^q, q such that every row sums to less than 2^60 in magnitude (by a margin
+            // that rounding and one entry's high part, an int, leave alone)
             double most = 0.0;
             for (int i = 0; i < n; ++i) {
                 double sum = 0.0;
                 for (int j = 0; j < bw; ++j) sum += fabs(hv[(size_t)i * bw + j]);
                 most = fmax(most, sum);
             }
-            c->sem_q = 57 - ilogb(most);
+            c->sem_q = 59 - ilogb(most * (1.0 + 0x1p-20));
             std::vector<int2> hx((size_t)bw * n);
             for (int i = 0; i < n; ++i)
                 for (int j = 0; j < bw; ++j) {

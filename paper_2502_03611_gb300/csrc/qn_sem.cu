@@ -13,8 +13,8 @@
 // A_h = sum over axes of H applied along that axis. H is banded (a node couples to
 // the nodes of its one or two elements): row i holds hlen[i] <= 2k+1 values from
 // column hc0[i]. One thread per node. k_residual_sem sums in FP64; the split solve's iterations
-// after the first take k_residual_sem_fixed, which forms the banded sums exactly from 57-bit
-// fixed-point values and coefficients on the integer pipe.
+// after the first take k_residual_sem_fixed, which forms the banded sums from 58-bit fixed-point
+// values and 61-bit coefficients on the integer pipe, exactly but for their roundings.
 #include <math.h>
 #include <string.h>
 
@@ -214,14 +214,29 @@ __global__ void __launch_bounds__(256) k_residual_sem(ResidualArgs a) {
 // ---- the banded sums on the integer pipe ------------------------------------------------
 // The FP64 kernel above is bound by the FP64 pipe (2 lanes per clock per SM): about 21 multiply-
 // adds along the axes and 11 other operations a node at Q^4, 1.03 ms at 255^3. Here every value
-// is an integer X = U 2^(1080 - E) with |X| < 2^56 (E two above the exponent of max|U|, taken by a
-// scan of U first) and every coefficient an integer C = H 2^q whose rows sum to at most 2^58 in
-// magnitude. Both are held as h 2^29 + l with |l| <= 2^28, and a tap is three 32 x 32 + 64-bit
-// multiply-adds: h h' and h l' + l h'. The l l' that are left out have zero mean and are below
-// 2^-57 of the largest value times the row sum together, where a chain of FP64 multiply-adds
-// rounds every partial sum at 2^-53; the two sums join in one 64-bit value that is rounded to
-// FP64 once. The limits hold for all degrees (3 x 33 taps at Q^16).
+// is an integer X = U 2^(1080 - E), rounded, with |X| <= 2^57 (E one above the exponent of max|U|,
+// taken by a scan of U first) and every coefficient an integer C = H 2^q, rounded, whose rows sum to
+// less than 2^60 in magnitude. Both are held as h 2^29 + l with |l| <= 2^28, and a tap is four
+// 32 x 32 + 64-bit multiply-adds: h h', h l' + l h' and l l'. The three sums join in one 64-bit value
+// that is rounded to FP64 once. The limits hold for all degrees (3 x 33 taps at Q^16: 2^61.6,
+// 2^62.95, 2^62.7). So the sums of the integers are exact, and their error is that of the roundings of
+// U and H: 2^-58 max|U| and 2^-60 to 2^-61 of the largest row sum a term. Over Q^1 to Q^16 the RMS
+// error of a sum is 0.01 to 0.5 of a chain of FP64 multiply-adds' on smooth and nearly constant
+// fields, 0.2 to 0.7 on noise, 0.3 to 1.1 on values from 1 to 1e-8; a single node whose neighbours are
+// all far below max|U| may be further off. (With the l l' left out and coefficients two
+// bits shorter the chains were closer from Q^6 on, by up to 3.9 at Q^16.)
 constexpr int kSemLo = 29;
+
+// As fx_of, rounded to nearest instead of cut; |v| <= 2^57 with E one above the exponent of max|U|.
+__device__ __forceinline__ long long sem_fixed(unsigned long long b, int E) {
+    const unsigned sh = (unsigned)(E - (int)((b >> 52) & 0x7FF));   // at least 1; zeros and subnormals shift out
+    const unsigned long long m = ((b & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << kFxG;
+    unsigned long long half, v;
+    asm("shl.b64 %0, %1, %2;" : "=l"(half) : "l"(1ull), "r"(sh - 1u));
+    asm("shr.b64 %0, %1, %2;" : "=l"(v) : "l"(m + half), "r"(sh));
+    const unsigned long long sg = (unsigned long long)((long long)b >> 63);   // 0 or all ones
+    return (long long)((v ^ sg) - sg);
+}
 
 __device__ __forceinline__ int2 sem_pair(long long v) {
     const int h = (int)((v + (1ll << (kSemLo - 1))) >> kSemLo);
@@ -231,18 +246,23 @@ __device__ __forceinline__ int2 sem_pair(long long v) {
 __global__ void __launch_bounds__(256) k_sem_to_fixed(const double *__restrict__ U, long long N, int2 *__restrict__ X,
                                                       const DevState *__restrict__ st) {
     if (*(volatile const int *)&st->done || st->fx_e == 0) return;
-    const int E = st->fx_e - st->fx_headroom + 2;
-    unsigned bad = 0;
+    const int E = st->fx_e - st->fx_headroom + 1;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
-        X[i] = sem_pair(fx_of((unsigned long long)__double_as_longlong(__ldg(U + i)), E, bad));
+        X[i] = sem_pair(sem_fixed((unsigned long long)__double_as_longlong(__ldg(U + i)), E));
 }
 
 struct SemSum {
     long long hh, mid;
+    long long ll;
     __device__ __forceinline__ void add(int2 x, int2 c) {
         hh += (long long)x.x * c.x;
         mid += (long long)x.x * c.y;
         mid += (long long)x.y * c.x;
+        ll += (long long)x.y * c.y;
+    }
+    // sum / 2^56
+    __device__ __forceinline__ long long total() const {
+        return (hh << 2) + ((mid + (ll >> 29) + (1ll << 26)) >> 27);
     }
 };
 
@@ -251,8 +271,9 @@ struct SemSum {
 // coefficients of the group sit in shared memory. KIND 0: general; 1: with a potential; 2:
 // lam = 0 and b = 1 (two FP64 operations a node fewer).
 //
-// Measured at 255^3, Q^4: 0.46 ms with four rows and four blocks per SM (64 registers, 80 bytes
-// spilled), 0.51 with three blocks, 0.48 with two rows; plus 0.07 ms for the scan and the
+// Measured at 255^3, Q^4, with three multiply-adds a tap: 0.46 ms with four rows and four blocks per
+// SM, 0.51 with three blocks, 0.48 with two rows; the fourth adds 4 % (a solve 10.7 -> 11.0 ms, and
+// 11.4 with three blocks per SM, 11.3 with l l' as high halves in 32 bits); plus 0.07 ms for the scan and the
 // conversion, against 1.03 ms in FP64. It waits on L1 / L2 loads of the neighbours' values.
 constexpr int kSemRows = 4, kSemBlocks = 4;   // blocks per SM
 
@@ -265,7 +286,7 @@ __global__ void __launch_bounds__(256, kSemBlocks) k_residual_sem_fixed(const Re
     const int n = a.n, P = a.P, bw = a.hbw;
     const int groups = (P / kSemRows) * ((DIM == 3) ? P : 1);   // P is a multiple of 64
     const int nn = n * n;                                        // n <= 1024
-    const int E = *a.fx_e - *a.fx_headroom + 2;
+    const int E = *a.fx_e - *a.fx_headroom + 1;
     const int2 *__restrict__ X = a.sem_x;
     const int2 *__restrict__ H = a.sem_h;   // [tap][row]
     Red4s acc{0.0, 0.0, INFINITY, -INFINITY};
@@ -339,8 +360,7 @@ __global__ void __launch_bounds__(256, kSemBlocks) k_residual_sem_fixed(const Re
 #pragma unroll
                 for (int r = 0; r < kSemRows; ++r) {
                     if (y0 + r >= n) break;
-                    // sum / 2^54, in units of 2^(E - 1026 - q)
-                    const double lap = fixed_to_double((s[r].hh << 4) + ((s[r].mid + (1ll << 24)) >> 25), E + 54 - a.sem_q);
+                    const double lap = fixed_to_double(s[r].total(), E + 56 - a.sem_q);   // units of 2^(E - 1024 - q)
                     const double u2 = u[r] * u[r];
                     double v;
                     if (KIND == 2) {
