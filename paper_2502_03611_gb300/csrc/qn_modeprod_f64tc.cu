@@ -36,6 +36,7 @@
 #include <cuda_fp16.h>
 #include <cudaTypedefs.h>
 #include <limits.h>
+#include <stdlib.h>
 #include <string.h>
 
 #include <new>
@@ -747,11 +748,14 @@ int f64tc_create(F64TcPlan **out, int n, int dim, int split, const double *S, co
         p->BN /= 2;
     p->ntn = (p->nrow + p->BN - 1) / p->BN;
     // rows per pass: the digits take 14 bytes per padded value, at most 2 GiB of them at a time
-    // (all rows up to 520^3; passes of 96 MB, which would stay in L2, lost more to the tails
-    // of their launches than they saved: 1.87 against 1.63 ms per 255^3 inverse)
-    long long ct = (2ll << 30) / ((long long)kDig * p->ld * 2 * BM);
+    // (QN_DIGIT_MB: another limit; all rows up to 520^3; passes of 96 MB, which would stay in L2,
+    // lost more to the tails of their launches than they saved: 1.87 against 1.63 ms per 255^3
+    // inverse), and less where the device has no room for that
+    const char *em = getenv("QN_DIGIT_MB");
+    const long long mb = (em && atoll(em) >= 1 && atoll(em) <= 2048) ? atoll(em) : 2048;
+    long long ct = (mb << 20) / ((long long)kDig * p->ld * 2 * BM);
+    if (ct < 1) ct = 1;
     if (ct > mtiles) ct = mtiles;
-    p->chunk = (int)ct * BM;
 
     auto fail = [&](int rc) {
         f64tc_destroy(p);
@@ -762,8 +766,17 @@ int f64tc_create(F64TcPlan **out, int n, int dim, int split, const double *S, co
     if (rc == QN_OK) rc = opt_in_bn<16>();
     if (rc != QN_OK) return fail(rc);
     CUtensorMap h[3];
-    if (cudaMalloc(&p->adig, (size_t)kDig * p->chunk * p->ld * 2) != cudaSuccess ||
-        cudaMalloc(&p->ea, sizeof(int2) * p->chunk) != cudaSuccess ||
+    while (cudaMalloc(&p->adig, (size_t)kDig * ct * BM * p->ld * 2) != cudaSuccess) {
+        p->adig = nullptr;
+        cudaGetLastError();
+        if (ct == 1) {
+            set_error("qn_ctx_create: out of device memory for the FP64 products' digits");
+            return fail(QN_ENOMEM);
+        }
+        ct = (ct + 1) / 2;
+    }
+    p->chunk = (int)ct * BM;
+    if (cudaMalloc(&p->ea, sizeof(int2) * p->chunk) != cudaSuccess ||
         cudaMalloc(&p->maps, sizeof(h)) != cudaSuccess) {
         set_error("qn_ctx_create: out of device memory for the FP64 products' digits");
         return fail(QN_ENOMEM);

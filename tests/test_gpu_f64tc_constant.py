@@ -1,4 +1,6 @@
-"""FP64 digit products whose digits repeat in every term: the constant row of the Neumann basis on
+"""FP64 digit products on fields that are not noise, and in passes.
+
+Fields whose digits repeat in every term: the constant row of the Neumann basis on
 fields that are constant up to 1e-7, where a sum of d + 1 digit products grows with the number of
 terms instead of averaging out. The inverse keeps the bound of any other field: 2 d products, each
 within 4 sqrt(n) roundings of its largest terms.
@@ -40,3 +42,23 @@ def test_near_constant_fields(dim, n, sem, rows):
                 X = X / (sum(lam.reshape([-1 if a == b else 1 for b in range(dim)]) for a in range(dim)) + 7.0)
         err = float(np.abs(V.cpu().numpy() - X).max() / np.abs(X).max())
         assert err <= 2 * dim * 4.0 * np.sqrt(n) * 2.0 ** -52, (c, err)
+
+
+@pytest.mark.parametrize("dim,n", [(3, 97), (3, 130), (2, 1001)])
+def test_passes_over_the_rows(monkeypatch, dim, n):
+    """Digits of a part of the rows at a time (little memory): the same bits."""
+    import torch
+
+    from paper_2502_03611_gb300 import qn
+    qn.load_library()
+    r = torch.from_numpy(np.random.default_rng(n).standard_normal((n,) * dim)).cuda()
+    outs = []
+    for mb in (None, "1", "7"):
+        if mb is None:
+            monkeypatch.delenv("QN_DIGIT_MB", raising=False)
+        else:
+            monkeypatch.setenv("QN_DIGIT_MB", mb)
+        V = torch.empty_like(r)
+        qn.qn_fast_diag_solve(qn.QnContext(dim, n, "fp64"), r, V, 7.0)
+        outs.append(V)
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
