@@ -44,6 +44,28 @@ def test_near_constant_fields(dim, n, sem, rows):
         assert err <= 2 * dim * 4.0 * np.sqrt(n) * 2.0 ** -52, (c, err)
 
 
+# values over eight decades and one node a billion times the others, within every row: the digits cut
+# each value at 2^-61 of its row's largest
+@pytest.mark.parametrize("n,bc", [(190, "dirichlet"), (255, "neumann"), (512, "dirichlet")])
+@pytest.mark.parametrize("field", ["wide", "spike"])
+def test_rows_of_wide_range(n, bc, field):
+    import torch
+
+    from paper_2502_03611_gb300 import qn
+    qn.load_library()
+    S, Si, lam = qn.qn_setup_1d_eig(n, 1.0 / (n + 1 if bc == "dirichlet" else n - 1), qn.BCS[bc])
+    rng = np.random.default_rng(n)
+    r = 10.0 ** rng.uniform(-8, 0, (n, n)) * rng.choice([-1.0, 1.0], (n, n))
+    if field == "spike":
+        r = 1e-9 * rng.standard_normal((n, n))
+        r[n // 2, n // 2] = 1.0
+    t = torch.from_numpy(r).cuda()
+    V = torch.empty_like(t)
+    qn.qn_fast_diag_solve(qn.QnContext(2, n, "fp64", bc=bc), t, V, 7.0)
+    X = S @ ((Si @ r @ Si.T) / (lam[:, None] + lam[None, :] + 7.0)) @ S.T
+    assert np.abs(V.cpu().numpy() - X).max() <= 4 * 4.0 * np.sqrt(n) * 2.0 ** -52 * np.abs(X).max()
+
+
 @pytest.mark.parametrize("dim,n", [(3, 97), (3, 130), (2, 1001)])
 def test_passes_over_the_rows(monkeypatch, dim, n):
     """Digits of a part of the rows at a time (little memory): the same bits."""
