@@ -423,7 +423,9 @@ long long qn_net_param_count(int channels, int modes, int blocks);
 
 /* Create a network on the current device. G: coarse grid nodes per axis
  * (2..256), channels == 32, modes in 1..min(G, 16), blocks 1..16,
- * max_batch 1..64 (activation buffers are sized for it). Parameters start at
+ * max_batch 1..64 (activation buffers are sized for it: with 2 to 8 modes 64 bytes per node and
+ * sample for each block's input, 64 for each block's z but the last's, 128 for the gradient and 8 for the
+ * outputs; other mode counts about 520 more for the unfused kernels). Parameters start at
  * zero: set them with qn_net_set_params. */
 int qn_net_create(int G, int channels, int modes, int blocks, int max_batch, qn_net **out);
 int qn_net_destroy(qn_net *net);

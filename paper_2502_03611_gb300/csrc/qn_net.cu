@@ -737,6 +737,10 @@ static void net_free(qn_net *n) {
         }                                     \
     } while (0)
 
+// The fused training kernels (qn_net_train.cuh) take 2 to 8 modes per axis.
+constexpr int kTrainMaxModes = 8;
+static bool net_fused(const qn_net *n) { return n->M >= 2 && n->M <= kTrainMaxModes; }
+
 static long long net_param_count(int C, int M, int L) {
     return 2LL * C + (long long)L * ((long long)M * M * M * C * C + (long long)C * C + C) + C + 1;
 }
@@ -785,36 +789,40 @@ extern "C" int qn_net_create(int G, int channels, int modes, int blocks, int max
     n->h.assign(blocks + 1, nullptr);
     n->z.assign(blocks, nullptr);
     n->hh.assign(blocks, nullptr);
-    for (int l = 0; l <= blocks; ++l) NCK(cudaMalloc(&n->h[l], sizeof(__nv_bfloat16) * act));
+    // what the fused kernels never store: the last block's z and output, and the unfused
+    // kernels' intermediates
+    const bool fused = net_fused(n);
+    for (int l = 0; l < blocks + (fused ? 0 : 1); ++l) NCK(cudaMalloc(&n->h[l], sizeof(__nv_bfloat16) * act));
     for (int l = 0; l < blocks; ++l) {
-        NCK(cudaMalloc(&n->z[l], sizeof(__nv_bfloat16) * act));
+        if (!fused || l < blocks - 1) NCK(cudaMalloc(&n->z[l], sizeof(__nv_bfloat16) * act));
         NCK(cudaMalloc(&n->hh[l], sizeof(float) * max_batch * K * channels));
     }
     // x-analysed tensor (unfused kernels), or the fused kernels' sums per plane and part
     const long long mp = (modes + 1) / 2 * 2;
-    long long tsz = (long long)max_batch * G * G * modes * channels;
-    if (tsz < (long long)max_batch * G * kTrParts * mp * mp * channels)
-        tsz = (long long)max_batch * G * kTrParts * mp * mp * channels;
-    NCK(cudaMalloc(&n->t1, sizeof(float) * tsz));
+    const long long tsz = fused ? (long long)max_batch * G * kTrParts * mp * mp * channels
+                                : (long long)max_batch * G * G * modes * channels;
     NCK(cudaMalloc(&n->t2, sizeof(float) * tsz));
-    NCK(cudaMalloc(&n->sp, sizeof(float) * act));
     NCK(cudaMalloc(&n->g, sizeof(float) * max_batch * K * channels));
-    NCK(cudaMalloc(&n->dg, sizeof(float) * max_batch * K * channels));
+    if (!fused) {
+        NCK(cudaMalloc(&n->t1, sizeof(float) * tsz));
+        NCK(cudaMalloc(&n->sp, sizeof(float) * act));
+        NCK(cudaMalloc(&n->dg, sizeof(float) * max_batch * K * channels));
+        NCK(cudaMalloc(&n->dz, sizeof(float) * act));
+        NCK(cudaMalloc(&n->dh2, sizeof(float) * act));
+        NCK(cudaMalloc(&n->tgt, sizeof(float) * pts));
+    }
     NCK(cudaMalloc(&n->dhh, sizeof(float) * max_batch * K * channels));
     NCK(cudaMalloc(&n->out, sizeof(float) * pts));
     NCK(cudaMalloc(&n->dout, sizeof(float) * pts));
     NCK(cudaMalloc(&n->dh, sizeof(float) * act));
-    NCK(cudaMalloc(&n->dz, sizeof(float) * act));
-    NCK(cudaMalloc(&n->dh2, sizeof(float) * act));
-    NCK(cudaMalloc(&n->fin, sizeof(float) * pts));
-    NCK(cudaMalloc(&n->tgt, sizeof(float) * pts));
+    NCK(cudaMalloc(&n->fin, sizeof(float) * (fused ? (long long)G * G * G : pts)));
     NCK(cudaMalloc(&n->loss, sizeof(double)));
     {
         const long long chunks = (G + kInfRows - 1) / kInfRows;
         NCK(cudaMalloc(&n->part, sizeof(float) * (size_t)(G * chunks * modes * modes * channels)));
         NCK(cudaMalloc(&n->wsq, 2 * sizeof(double)));
     }
-    if (modes >= 2 && modes <= 8) {
+    if (fused) {
         const int rc = modes <= 2 ? tr_set_attributes<2>()
                                   : (modes <= 4 ? tr_set_attributes<4>()
                                                 : (modes <= 6 ? tr_set_attributes<6>() : tr_set_attributes<8>()));
@@ -872,9 +880,6 @@ static long long off_wp(qn_net *n) { return block_base(n, n->L); }
 
 // Forward (and, with a target, loss and backward) through the fused kernels of
 // qn_net_train.cuh: 2 to 8 modes per axis. f, target: the caller's arrays, read in place.
-constexpr int kTrainMaxModes = 8;
-static bool net_fused(const qn_net *n) { return n->M >= 2 && n->M <= kTrainMaxModes; }
-
 static int net_fused_pass(qn_net *n, const float *f, const float *target, float *out, int B, cudaStream_t s) {
     long long oR[16], oW[16], ob[16];
     for (int l = 0; l < n->L; ++l) {
