@@ -683,7 +683,7 @@ inline int grid_axis(long long elements) { return grid_for((elements + axis_run(
 using namespace qn;
 
 struct qn_net {
-    int G, C, M, L, Bmax;
+    int G, C, M, L, Bmax, num_sms;
     long long nparams;
     float *params, *grads, *am, *av;
     float *basis_a;   // M x G (analysis: out[k] = sum_j B[j][k] in[j])
@@ -763,6 +763,9 @@ extern "C" int qn_net_create(int G, int channels, int modes, int blocks, int max
     n->M = modes;
     n->L = blocks;
     n->Bmax = max_batch;
+    int dev = 0;
+    NCK(cudaGetDevice(&dev));
+    NCK(cudaDeviceGetAttribute(&n->num_sms, cudaDevAttrMultiProcessorCount, dev));
     n->nparams = net_param_count(channels, modes, blocks);
     const long long pts = (long long)max_batch * G * G * G;
     const long long act = pts * channels;
@@ -888,7 +891,7 @@ static int net_fused_pass(qn_net *n, const float *f, const float *target, float 
         ob[l] = off_b(n, l);
     }
     TrNet t{n->G, n->M, n->L, B, f, target, n->basis_s, n->params, n->grads, n->t2, n->g, n->dhh, out, n->dout, n->dh,
-            n->loss, n->h.data(), n->z.data(), n->hh.data(), oR, oW, ob, off_wp(n)};
+            n->loss, n->h.data(), n->z.data(), n->hh.data(), oR, oW, ob, off_wp(n), n->num_sms};
     if (target != nullptr) {
         QN_CUDA(cudaMemsetAsync(n->grads, 0, sizeof(float) * n->nparams, s));
         QN_CUDA(cudaMemsetAsync(n->loss, 0, sizeof(double), s));

@@ -1,10 +1,11 @@
 // Training kernels of the warm-start network (forward, loss, backward) for up to eight modes per
 // axis. Included by qn_net.cu.
 //
-// A block's work is bound by HBM once nothing is read twice: an activation of 8 x 64^3 nodes is
-// 134 MB in BF16 and a gradient 268 MB in FP32. Per block l the kernels are
-//   k_tr_analysis   one read of h_l (or of dh and z_l): the x and y analysis of a z plane per
-//                   CTA, which writes M^2 x 32 sums a plane instead of the x-analysed tensor;
+// An activation of 8 x 64^3 nodes is 134 MB in BF16 and a gradient 268 MB in FP32, so nothing is
+// read twice; what is left waits on instruction issue (FP32 multiply-adds of the transforms,
+// 43 to 66 %) and shared memory, at 1 to 3 TB/s. Per block l the kernels are
+//   k_tr_analysis   one read of h_l (or of dh and z_l): the x and y analysis of a quarter of a z
+//                   plane per CTA, which writes M^2 x 32 sums instead of the x-analysed tensor;
 //   k_tr_mix        z analysis and channel mixing, one CTA per mode (backward: both gradients);
 //   k_tr_fwd        z_l = synthesis(g) + h_l W + b and h_{l+1}; the spectral term is formed in
 //                   registers per row. The last block also projects, takes the loss and its
@@ -876,6 +877,7 @@ struct TrNet {
     float *const *hh;
     const long long *off_R, *off_W, *off_b;
     long long off_wp;
+    int num_sms;   // two (forward) and three (backward) resident CTAs on each
 };
 
 template <typename K>
@@ -906,7 +908,7 @@ template <int MP>
 void tr_forward(const TrNet &n, cudaStream_t s) {
     const int planes = n.B * n.G, K = n.M * n.M * n.M;
     const int items = planes * ((n.G + kTrRows - 1) / kTrRows);
-    const int grid = items < 2 * 152 ? items : 2 * 152;
+    const int grid = items < 2 * n.num_sms ? items : 2 * n.num_sms;
     for (int l = 0; l < n.L; ++l) {
         TrFwd a{};
         a.in.h = n.h[l];
@@ -951,7 +953,7 @@ template <int MP>
 void tr_backward(const TrNet &n, cudaStream_t s) {
     const int planes = n.B * n.G, K = n.M * n.M * n.M;
     const int items = planes * ((n.G + kTrRows - 1) / kTrRows);
-    const int grid = items < 3 * 152 ? items : 3 * 152;
+    const int grid = items < 3 * n.num_sms ? items : 3 * n.num_sms;
     for (int l = n.L - 1; l >= 0; --l) {
         const bool last = l == n.L - 1;
         TrBwd a{};
