@@ -634,18 +634,21 @@ def run_c2(qn, seeds=(0, 1, 2), want_cpu=True):
     flops = (1.0 if split else 2.0) * float(n) ** 4
     tfl = flops / (mp_ms * 1e-3) / 1e12
     dg = dgemm_tflops(stream)
+    peaks, peak_src = load_peaks()
+    peak = float(peaks.get("bf16_tflops_sustained", FALLBACK_PEAKS["bf16_tflops_sustained"]))
     tot = prof["residual_ms"] + prof["modeprod_ms"] + prof["finalize_ms"]
     out = {"workload": "3-D -Lap u + u^3 = f, 255^3 interior, 7-point FD, Dirichlet 0, FP64 throughout, "
                        f"zero start, tol 1e-10, seeds {list(seeds)}",
            "precision": "fp64", "ms_per_solve_median": round(statistics.median(ms), 2),
            "ms_per_solve": [round(m, 2) for m in ms], "iterations": its,
-           # FP64 results from FP16 digit products on the tensor cores: the FP64 pipe's DGEMM rate
-           # is what they replace, so the fraction is far above one
-           "roofline": {"kernel": "k_modeprod_f64tc + k_slice_rows", "bound": "tensor + hbm", "achieved": round(tfl, 4),
-                        "peak": round(dg, 4), "unit": "TFLOP/s", "frac": round(tfl / dg, 4),
-                        "executed_fp16_tflops": round(28 * tfl, 1),
-                        "peak_source": "cuBLAS DGEMM 4096^3 measured in this run (the FP64 pipe, which the "
-                                       "products do not use)",
+           # FP64 results from 28 FP16 digit products on the tensor cores: their rate over a launch
+           # (the slicing of the rows included) against the 16-bit tensor rate
+           "roofline": {"kernel": "k_modeprod_f64tc + k_slice_rows", "bound": "tensor",
+                        "achieved": round(28 * tfl, 1), "peak": peak, "unit": "TFLOP/s (executed, FP16 digits)",
+                        "frac": round(28 * tfl / peak, 4), "peak_source": f"bf16 dense, sustained ({peak_src})",
+                        "fp64_tflops": round(tfl, 4), "times_dgemm": round(tfl / dg, 2), "dgemm_tflops": round(dg, 4),
+                        "dgemm_source": "cuBLAS 4096^3 measured in this run (the FP64 pipe, which the products "
+                                        "do not use)",
                         "split_products": split, "flops_per_launch_algorithmic": flops,
                         "avg_launch_ms": round(mp_ms, 4), "launches": prof["modeprod_launches"],
                         "share": round(prof["modeprod_ms"] / tot, 4) if tot else None},
@@ -1045,19 +1048,21 @@ def main():
     barrier()
     torch.cuda.synchronize()
     sampler.start()
-    ev0 = torch.cuda.Event(enable_timing=True)
-    ev1 = torch.cuda.Event(enable_timing=True)
-    ev0.record(stream)
+    marks = [torch.cuda.Event(enable_timing=True) for _ in range(a.steps + 1)]
+    marks[0].record(stream)
     results = []
-    for _ in range(a.steps):
+    for k in range(a.steps):
         reset_start()
         res, _ = qn.qn_solve(ctx, U, f, max_it=max_it, graph=True)
         results.append(res)
-    ev1.record(stream)
+        marks[k + 1].record(stream)
     torch.cuda.synchronize()
     barrier()
     clocks = sampler.stop()
-    elapsed_ms = ev0.elapsed_time(ev1)
+    elapsed_ms = marks[0].elapsed_time(marks[-1])
+    # the steps one by one: a stall of the host shows as a maximum far above the median
+    each = [x.elapsed_time(y) for x, y in zip(marks, marks[1:])] or [elapsed_ms]
+    spread = {"min": round(min(each), 3), "median": round(statistics.median(each), 3), "max": round(max(each), 3)}
     timed_launches = int(qn.qn_profile_read(ctx)["launches"])
     # the last timed solve's result, for the comparison with the oracle (after the GPU legs)
     U_result = U.cpu().numpy().copy() if (not a.no_cpu and rank == 0 and world == 1
@@ -1098,9 +1103,9 @@ def main():
         peak = None
         peak_name = "fp64 (see plain_fp64.fp64_peak)"
     kernel_file = os.path.join(ROOT, "paper_2502_03611_gb300", "csrc",
-                               "qn_modeprod_tc.cu" if a.precision == "bf16x3" else "qn_modeprod_f64.cu")
+                               "qn_modeprod_tc.cu" if a.precision == "bf16x3" else "qn_modeprod_f64tc.cu")
     traffic = ncu_traffic(kernel_file) if a.precision == "bf16x3" else None
-    tensor_roofline = {"kernel": "k_modeprod_tc" if a.precision == "bf16x3" else "k_modeprod_f64",
+    tensor_roofline = {"kernel": "k_modeprod_tc" if a.precision == "bf16x3" else "k_modeprod_f64tc",
                        "bound": "tensor", "achieved": round(mp_tflops, 2), "peak": peak, "unit": "TFLOP/s",
                        "frac": round(mp_tflops / peak, 4) if peak else None,
                        "peak_source": peak_name, "split_products": split,
@@ -1368,10 +1373,11 @@ def main():
         del Uo
 
     if rank == 0 and sem:
-        # the SEM residual is bound by instruction issue (integer band sums in split precision) or
-        # the FP64 pipe (FP64 contexts): algorithmic FLOP per launch = per node
-        # 2 x (band entries of H along each axis) + 9 for the nonlinear term and the norm, against
-        # a cuBLAS DGEMM measured here (no FP64 peak is in MEASURED_PEAKS)
+        # the SEM residual of a split-precision solve (integer band sums) is bound by instruction
+        # issue: achieved and peak are its algorithmic bytes (U, f and the two planes) over HBM. In FP64
+        # contexts it is bound by the FP64 pipe: algorithmic FLOP per launch = per node 2 x (band entries of H
+        # along each axis) + 9 for the nonlinear term and the norm, against a cuBLAS DGEMM measured here (no
+        # FP64 peak is in MEASURED_PEAKS), which the other form reports as times_dgemm
         Hm = qn.qn_setup_1d_sem(n, a.sem_k, 1.0, qn.QN_BC_DIRICHLET)[0]
         avg_nnz = float(np.count_nonzero(Hm)) / n
         flops_res = N * (2.0 * 3 * avg_nnz + 9.0)
@@ -1391,16 +1397,23 @@ def main():
         dgemm = 5 * 2 * 4096.0 ** 3 / (g0.elapsed_time(g1) * 1e-3) / 1e12
         del A, B
         ach = flops_res / (res_ms * 1e-3) / 1e12
-        roofline = {"kernel": "k_residual_sem" if a.precision == "fp64" else "k_residual_sem_fixed",
-                    "bound": "fp64" if a.precision == "fp64" else "issue", "achieved": round(ach, 4), "peak": round(dgemm, 4),
-                    "unit": "TFLOP/s", "frac": round(ach / dgemm, 4), "traffic": None,
-                    "peak_source": "cuBLAS DGEMM 4096^3 measured in this run (FP64 pipe)",
+        dgemm_src = "cuBLAS DGEMM 4096^3 measured in this run (FP64 pipe)"
+        if a.precision == "fp64":
+            roofline = {"kernel": "k_residual_sem", "bound": "fp64", "achieved": round(ach, 4), "peak": round(dgemm, 4),
+                        "unit": "TFLOP/s", "frac": round(ach / dgemm, 4), "peak_source": dgemm_src}
+        else:
+            gbs = (16.0 * N + 4.0 * float(P) ** 3) / (res_ms * 1e-3) / 1e9
+            roofline = {"kernel": "k_residual_sem_fixed", "bound": "issue", "achieved": round(gbs, 1),
+                        "peak": round(hbm, 1), "unit": "GB/s", "frac": round(gbs / hbm, 4),
+                        "peak_source": f"HBM copy bandwidth ({peak_src})", "algorithmic_tflops": round(ach, 4),
+                        "times_dgemm": round(ach / dgemm, 2), "dgemm_source": dgemm_src}
+        roofline = {**roofline, "traffic": None,
                     "flops_per_launch_algorithmic": flops_res, "band_entries_per_row": round(avg_nnz, 3),
                     "avg_launch_ms": round(res_ms, 4), "launches": prof["residual_launches"]}
         line = {
             "metric": "time to rel. residual 1e-10, 3-D Q^k spectral elements at n^3 nodes", "value": round(ms_max, 3),
             "unit": "ms", "n_gpus": world, "steps": a.steps, "warmup": a.warmup, "ms_per_step": round(ms_max, 3),
-            "higher_is_better": False, "scaling": "weak", "vs_baseline": None,
+            "ms_each_step": spread, "higher_is_better": False, "scaling": "weak", "vs_baseline": None,
             "dtype": "bf16x3+f64" if a.precision == "bf16x3" else "f64",
             "data": "synthetic (closed-form source of u* = sin(pi x) sin(pi y) sin(pi z) at the nodes)",
             "config": {"workload": f"3-D -Lap u + u^3 = f on (0,1)^3, Q^{a.sem_k} spectral elements (Gauss-Lobatto, "
@@ -1419,7 +1432,7 @@ def main():
         line = {
             "metric": METRIC_EX1, "value": round(ms_max, 3), "unit": "ms", "n_gpus": world,
             "steps": a.steps, "warmup": a.warmup, "ms_per_step": round(ms_max, 3),
-            "higher_is_better": False, "scaling": "weak", "vs_baseline": None,
+            "ms_each_step": spread, "higher_is_better": False, "scaling": "weak", "vs_baseline": None,
             "dtype": "bf16x3+f64" if a.precision == "bf16x3" else "f64",
             "data": "synthetic (closed-form source of u* = cos(pi x)+cos(pi y)+cos(pi z); seed-drawn "
                     "start perturbation)",
@@ -1444,7 +1457,7 @@ def main():
         line = {
             "metric": METRIC, "value": round(ms_max, 3), "unit": "ms", "n_gpus": world,
             "steps": a.steps, "warmup": a.warmup, "ms_per_step": round(ms_max, 3),
-            "higher_is_better": False, "scaling": "weak", "vs_baseline": None,
+            "ms_each_step": spread, "higher_is_better": False, "scaling": "weak", "vs_baseline": None,
             "dtype": ("bf16x3 products (fp32 accumulate); int64 fixed-point + fp32-pair residual; f64 update"
                       if a.precision == "bf16x3" else "f64"),
             "data": "synthetic (manufactured sine-series source, 6x6x6 modes, seed-drawn)",
