@@ -69,9 +69,10 @@ extern "C" {
                                finite differences, per-node residual kernel */
 
 #define QN_PREC_FP64   0    /* mode products of FP64 operands with FP64 results: n^(dim+1) above
-                               6e6 as exact integer digits on the tensor cores (seven nine-bit
-                               digits per value, rounded at the end; closer to the exact product
-                               than a chain of FP64 multiply-adds), smaller ones on the FP64 pipe */
+                               6e6 as integer digits on the tensor cores (seven nine-bit digits per
+                               value, each value cut at 2^-61 of the largest of its row, rounded at
+                               the end; an inverse is closer to the exact one than with chains of
+                               FP64 multiply-adds), smaller ones on the FP64 pipe */
 #define QN_PREC_BF16X3 1    /* mode products on tcgen05 tensor cores as
                                hi*hi + hi*lo + lo*hi BF16 products, FP32
                                accumulation; residual, beta, update and stop
@@ -196,8 +197,9 @@ int qn_setup_1d_sem(int n, int k, double length, int bc, double *H, double *S, d
  * S, S^{-1} and the eigenvalues (and their BF16 hi/lo splits for
  * QN_PREC_BF16X3 / BF16X6), allocates the working buffers (about 2 n^dim doubles for
  * FP64, where the products run on the tensor cores with the digits of one operand besides:
- * 14 bytes per value, at most 2 GiB at a time; 2 padded n^dim x 4 bytes for BF16X3) and, for BF16X3, builds the TMA
- * tensor maps. QN_EUNSUPPORTED for BF16X3 on a device without sm_103a
+ * 14 bytes per value, at most 2 GiB at a time and less where the device has no room; 2 padded
+ * n^dim x 4 bytes for BF16X3, with sem_k > 0 another 8 n^dim for the fixed-point U of the
+ * residual) and, for BF16X3, builds the TMA tensor maps. QN_EUNSUPPORTED for BF16X3 on a device without sm_103a
  * tcgen05 support. *out is owned by the library until qn_ctx_destroy. */
 int qn_ctx_create(const qn_problem *p, qn_ctx **out);
 
@@ -514,7 +516,10 @@ typedef struct qn_profile {
     double residual_tiled_ms;
     int split_products;       /* 1: the last shifted inverse used the reflection-split mode
                                  products (3-D split solve; P = 64 ceil(n/64) a multiple of
-                                 128, or at least 320): half the tensor work of the dense products */
+                                 128, or at least 320): half the tensor work of the dense products.
+                                 FP64 contexts: 1 when the context's products use the symmetry
+                                 (sine or cosine basis, QN_SPLIT not 0), also at sizes whose products
+                                 are so small that the dense kernel forms them */
     int x6_from;              /* the last qn_solve: the first iteration whose backward products
                                  ran at the six-product level (0 in a QN_PREC_BF16X6 context,
                                  the escalation point after qn_set_escalation), -1: none */
